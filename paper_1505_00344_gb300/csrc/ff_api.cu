@@ -82,10 +82,7 @@ ff_status seed_group(ff_system* s, const Group& g) {
     a.first = g.first;
     a.seed = g.seed;
     a.dim = s->dim;
-    for (int k = 0; k < s->dim; ++k) {
-        a.lo[k] = g.lo[k];
-        a.width[k] = g.hi[k] - g.lo[k];
-    }
+    for (int k = 0; k < s->dim; ++k) a.box[k] = ff::draw_box(g.lo[k], g.hi[k]);
     cudaError_t e = ff::launch_seed(a, s->num_sms, s->stream);
     if (e != cudaSuccess) return cuda_fail(e, "seed kernel launch");
     return FF_OK;
@@ -418,10 +415,7 @@ static ff_status upload_reset_table(ff_system* s) {
     ff::ResetTable& t = s->h_reset_table;
     t = ff::ResetTable{};
     for (int g = 0; g < s->n_groups; ++g) {
-        for (int k = 0; k < s->dim; ++k) {
-            t.lo[g][k] = s->groups[g].lo[k];
-            t.width[g][k] = s->groups[g].hi[k] - s->groups[g].lo[k];
-        }
+        for (int k = 0; k < s->dim; ++k) t.box[g][k] = ff::draw_box(s->groups[g].lo[k], s->groups[g].hi[k]);
         t.count[g] = s->groups[g].total;
         t.first[g] = s->groups[g].first;
         t.seed[g] = s->groups[g].seed;

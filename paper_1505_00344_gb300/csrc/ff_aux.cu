@@ -11,28 +11,16 @@ namespace ff {
 
 // ---------------------------------------------------------------------------
 // Seeding (paper Appendix A, "Particle Group" / "Initialization").
-// SplitMix64 (Steele, Lea & Flood 2014): output n of the stream seeded with s
-// is the variant-13 finaliser applied to s + n * 0x9E3779B97F4A7C15.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint64_t n) {
-    uint64_t z = seed + n * 0x9E3779B97F4A7C15ULL;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
-    return z ^ (z >> 31);
-}
-
-// Group particle j, variable k: draw n = j*dim + k + 1; u = top 24 bits / 2^24;
-// x = lo + width * u in double (separately rounded), then to nearest float.
+// Group particle j, variable k: draw n = j*dim + k + 1 of the group's stream (draw_value).
+// Bound by the integer pipe (two 64-bit multiplications per value) and the 4 bytes written.
 __global__ void seed_kernel(const __grid_constant__ SeedArgs a) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < a.count; j += stride) {
         const uint64_t jg = (uint64_t)(a.first + j);  // index within the whole group
-        for (int k = 0; k < a.dim; ++k) {
-            const uint64_t r = splitmix64_at(a.seed, jg * (uint64_t)a.dim + (uint64_t)k + 1u);
-            const double u = (double)(r >> 40) * (1.0 / 16777216.0);
-            const double v = __dadd_rn(a.lo[k], __dmul_rn(a.width[k], u));
-            a.x[k * a.pitch + a.start + j] = __double2float_rn(v);
-        }
+        uint64_t z = a.seed + (jg * (uint64_t)a.dim + 1u) * kSplitMixGamma;
+        for (int k = 0; k < a.dim; ++k, z += kSplitMixGamma)
+            a.x[k * a.pitch + a.start + j] = draw_value(splitmix64_mix(z), a.box[k]);
     }
 }
 

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "ff.h"
+#include "ff_draw.cuh"
 #include "ff_project.cuh"
 
 namespace ff {
@@ -18,8 +19,7 @@ struct SeedArgs {
     uint64_t seed;
     int dim;
     int pad_;
-    double lo[FF_MAX_DIM];
-    double width[FF_MAX_DIM];  // hi - lo, formed in double on the host
+    DrawBox box[FF_MAX_DIM];
 };
 
 constexpr int kSplatBlock = 256;

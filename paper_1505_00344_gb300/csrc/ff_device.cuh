@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "ff.h"
+#include "ff_draw.cuh"
 #include "ff_project.cuh"
 
 namespace ff {
@@ -107,22 +108,13 @@ __device__ __forceinline__ void run_steps(const IntegrateArgs& a, int n_steps, S
 
 // Reset data of a system, in device memory (read only when a particle resets).
 struct ResetTable {
-    double lo[FF_MAX_GROUPS][FF_MAX_DIM];
-    double width[FF_MAX_GROUPS][FF_MAX_DIM];  // hi - lo in double, as for the initial seeding
+    DrawBox box[FF_MAX_GROUPS][FF_MAX_DIM];
     int64_t count[FF_MAX_GROUPS];             // particles of the whole group (a slice's is its group's)
     int64_t first[FF_MAX_GROUPS];             // index within the whole group of the group's first particle
     uint64_t seed[FF_MAX_GROUPS];
     float blo[FF_MAX_DIM], bhi[FF_MAX_DIM];
     int has_bounds;
 };
-
-// SplitMix64 output n of the stream seeded with s (Steele, Lea & Flood 2014).
-__device__ __forceinline__ uint64_t reset_splitmix64(uint64_t seed, uint64_t n) {
-    uint64_t z = seed + n * 0x9E3779B97F4A7C15ULL;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
-    return z ^ (z >> 31);
-}
 
 // ---------------------------------------------------------------------------
 // Right-hand sides.  Each has DIM (registers per particle state), NP (params)
@@ -641,9 +633,7 @@ __device__ __forceinline__ void reset_check(const IntegrateArgs& a, const Steppe
 #pragma unroll
     for (int k = 0; k < D; ++k) {
         if (k < a.dim) {
-            const uint64_t z = reset_splitmix64(t->seed[g], base + (uint64_t)k + 1u);
-            const double u = (double)(z >> 40) * (1.0 / 16777216.0);
-            e[k] = __double2float_rn(__dadd_rn(t->lo[g][k], __dmul_rn(t->width[g][k], u)));
+            e[k] = draw_value(splitmix64_mix(t->seed[g] + (base + (uint64_t)k + 1u) * kSplitMixGamma), t->box[g][k]);
         } else {
             e[k] = 0.0f;
         }

@@ -40,3 +40,32 @@ def test_parameter_gradient_sums_every_partial_row(n):
     parts = sum(grad(a, b - a) for a, b in zip(cuts, cuts[1:]))
     whole = grad(0, n)
     assert abs(whole - parts) <= 1e-9 * abs(whole)
+
+
+# Boxes at the edges of the pair arithmetic of the draws: ordinary ones, intervals far from
+# zero, across zero, of width zero, much narrower than their offset, at and beyond the scales
+# that take the double formula, and bounds that are no floats.
+BOXES = [(0.0, 1.0), (-30.0, 30.0), (-80.0, 40.0), (0.1, 0.30000000000000004), (1e6, 1e6 + 1e-3), (-1e-3, 1e6),
+         (3.0, 3.0), (0.0, 0.0), (-0.0, 1e-11), (-1e-13, 1e-13), (2.0**-42, 2.0**-41), (-1e30, 1e30), (-1e31, 2e31),
+         (-3e38, 3e38), (1.0, 1.0 + 2.0**-23), (-1.0 / 3.0, 2.0 / 3.0)]
+
+
+@pytest.mark.parametrize("count", [1, 257, 40_003])
+def test_seeding_is_the_double_formula_for_every_box(count):
+    """x = fl32(lo + width * u), both double operations rounded, for u the top 24 bits of
+    SplitMix64 output j * dim + k + 1 -- bit for bit, whichever arithmetic formed it."""
+    with np.errstate(over="ignore"):
+        z = np.uint64(99) + np.arange(1, 2 * count + 1, dtype=np.uint64) * np.uint64(0x9E3779B97F4A7C15)
+        z = (z ^ (z >> np.uint64(30))) * np.uint64(0xBF58476D1CE4E5B9)
+        z = (z ^ (z >> np.uint64(27))) * np.uint64(0x94D049BB133111EB)
+        u = ((z ^ (z >> np.uint64(31))) >> np.uint64(40)).astype(np.float64) / 2.0 ** 24
+    u = u.reshape(count, 2).T
+    for a, b in zip(BOXES[0::2], BOXES[1::2]):
+        lo, hi = np.array([[a[0]], [b[0]]]), np.array([[a[1]], [b[1]]])
+        with np.errstate(over="ignore"):
+            want = (lo + (hi - lo) * u).astype(np.float32)
+        s = ff.System("harmonic", [1.0], count, stream=_stream())
+        s.seed(count, [a[0], b[0]], [a[1], b[1]], +1, 99)
+        got = np.empty((2, count), np.float32)
+        s.get_state(got)
+        np.testing.assert_array_equal(got.view(np.uint32), want.view(np.uint32), err_msg=f"{a} {b}")
