@@ -42,17 +42,14 @@ static_assert(kSplitBlockParticles == kAdjTileHH3, "one batched tile per block")
 __device__ __forceinline__ f2 mulp(f2 a, f2 b) { return mul2(a, b); }
 __device__ __forceinline__ f2 kp(float c) { return pack2(c, c); }
 
-__device__ __forceinline__ f2 lane_shfl(f2 v, int src) {
-    f2 r;
-    r.v = __shfl_sync(0xffffffffu, v.v, src);
-    return r;
-}
-
 // (v of neuron 0 + v of neuron 1) + v of neuron 2 over the lane's triple, the order of
 // HH3::f's sum of s.  src0 is the triple's first lane (lanes 30 and 31 read lanes 30, 31
 // and 0: whatever they get is discarded).
 __device__ __forceinline__ f2 triple_sum(f2 v, int src0) {
-    const f2 a = lane_shfl(v, src0), b = lane_shfl(v, src0 + 1), c = lane_shfl(v, src0 + 2);
+    f2 a, b, c;
+    a.v = __shfl_sync(0xffffffffu, v.v, src0);
+    b.v = __shfl_sync(0xffffffffu, v.v, src0 + 1);
+    c.v = __shfl_sync(0xffffffffu, v.v, src0 + 2);
     return add2(add2(a, b), c);
 }
 
@@ -105,10 +102,7 @@ __device__ __forceinline__ void lane_fwd(f2 (&X)[5], const LaneC& L, int src0, u
     } else {
         f2 XS[5], A[5];
 #pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            XS[k] = X[k];
-            A[k] = kp(0.0f);
-        }
+        for (int k = 0; k < 5; ++k) XS[k] = X[k];
         // the four stages unrolled (so are the reverse step's four products): each lane
         // holds one neuron, so there is room for the next stage's independent work in flight
 #pragma unroll
@@ -116,10 +110,8 @@ __device__ __forceinline__ void lane_fwd(f2 (&X)[5], const LaneC& L, int src0, u
             f2 K[5];
             hh_neuron<HHPair>(XS[0], XS[1], XS[2], XS[3], XS[4], sub2(triple_sum(XS[4], src0), XS[4]), L.driveC, L.c,
                               K);
-            const float w = (st == 1 || st == 2) ? 2.0f : 1.0f;  // fmaf(1, k, 0) = k
-            const f2 W = kp(w);
 #pragma unroll
-            for (int k = 0; k < 5; ++k) A[k] = fma2(W, K[k], A[k]);
+            for (int k = 0; k < 5; ++k) A[k] = rk4_weigh<HHPair>(st, K[k], A[k]);
             if (st == 3) break;
             const f2 C = (st == 2) ? L.H1 : L.H2;
 #pragma unroll

@@ -254,7 +254,6 @@ __device__ __forceinline__ typename O::T bernoulli_series_t(typename O::T y) {
                                         O::k(1.0f / 12.0f)), O::k(1.0f));
     return O::fma(O::k(0.5f), y, even);
 }
-__device__ __forceinline__ float bernoulli_series(float y) { return bernoulli_series_t<HHScalar>(y); }
 
 // Derivatives of one neuron: V, m, h, n, s its state, `others` the sum of the
 // other neurons' s, `driveC` its injected current divided by C (hh_drive_c).
@@ -274,7 +273,6 @@ __device__ __forceinline__ void hh_neuron(typename O::T V, typename O::T m, type
     const T q2 = O::mul(q, q), q4 = O::mul(q2, q2), q8 = O::mul(q4, q4);
     const T bm = O::ex2(O::fma(V, O::k(kB), O::k(kB0)));
     const T ah = O::mul(O::k(0.07f), q4);
-    const T bn = O::mul(O::k(0.125f), q);
     const T es = O::ex2(O::fma(c.neg_sig2, V, c.sig2_theta));  // e^(sig (theta - V))
     // alpha_m = g(ym), alpha_n = g(yn) / 10 with g(y) = y / (1 - e^-y),
     // ym = (V + 40) / 10, yn = (V + 55) / 10, e^-ym = e^2.5 q^8, e^-yn = e q^8
@@ -303,7 +301,7 @@ __device__ __forceinline__ void hh_neuron(typename O::T V, typename O::T m, type
     // toolchain would fuse the f32x2 form of an unfused product and difference anyway)
     d[1] = O::fms(O::add(am, bm), m, am);
     d[2] = O::fms(O::fma(ps, r, ah), h, ah);  // ah + bh with bh = ps r, fused likewise
-    d[3] = O::fms(O::add(an, bn), n, an);
+    d[3] = O::fms(O::fma(O::k(0.125f), q, an), n, an);  // beta_n = q / 8, an exact product
     d[4] = O::fma(O::mul(act, c.inv_tr), O::sub(one, s), O::mul(s, c.neg_inv_td));
 }
 
@@ -1267,6 +1265,12 @@ struct HHPair {
     __device__ __forceinline__ static T fms(T t, T y, T a) { return sub2(a, mul2(t, y)); }
 };
 
+// The weighted sum k1 + 2 k2 + 2 k3 + k4 after stage st (0..3; unrolled loops), a the sum before it.
+template <class O>
+__device__ __forceinline__ typename O::T rk4_weigh(int st, typename O::T k, typename O::T a) {
+    return st == 0 ? k : (st == 3 ? O::add(a, k) : O::fma(O::k(2.0f), k, a));
+}
+
 struct HH3RK4Packed {
     static constexpr int D = 15;
     float h1, h2, h6;
@@ -1290,10 +1294,8 @@ struct HH3RK4Packed {
         for (int k = 0; k < 5; ++k) {
             X[k] = pack2(x[k], x[5 + k]);
             XS[k] = X[k];
-            A[k] = pack2(0.0f, 0.0f);
             x2[k] = x[10 + k];
             xs2[k] = x2[k];
-            a2[k] = 0.0f;
         }
         // the stages unrolled: 4% faster than a stage loop (65,536 particles of hh3_1M)
 #pragma unroll
@@ -1303,12 +1305,10 @@ struct HH3RK4Packed {
             const float s_sum = __fadd_rn(__fadd_rn(s0, s1), xs2[4]);
             hh_neuron<HHPair>(XS[0], XS[1], XS[2], XS[3], XS[4], sub2(pack2(s_sum, s_sum), XS[4]), drive01, c2, K);
             hh_neuron<HHScalar>(xs2[0], xs2[1], xs2[2], xs2[3], xs2[4], __fsub_rn(s_sum, xs2[4]), drive2, c1, k2);
-            const float w = (st == 1 || st == 2) ? 2.0f : 1.0f;  // fmaf(1, k, 0) = k
-            const f2 W = pack2(w, w);
 #pragma unroll
             for (int k = 0; k < 5; ++k) {
-                A[k] = fma2(W, K[k], A[k]);
-                a2[k] = fmaf(w, k2[k], a2[k]);
+                A[k] = rk4_weigh<HHPair>(st, K[k], A[k]);
+                a2[k] = rk4_weigh<HHScalar>(st, k2[k], a2[k]);
             }
             if (st == 3) break;
             const float cst = (st == 2) ? h1 : h2;
@@ -1361,6 +1361,26 @@ __device__ __forceinline__ HHConst<HHPair> hh_const_pair(const float* pa, const 
     return c;
 }
 
+// Steps and parameter vectors of particles i0 and, with PER 2, i0 + 1 (PER 1: i0 twice).
+template <bool PP, int PER = 2>
+__device__ __forceinline__ void hh_pair_params(const IntegrateArgs& a, int64_t i0, float (&hs)[2],
+                                               float (&pa)[HH3::NP], float (&pb)[HH3::NP]) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int64_t i = i0 + j * (PER - 1);
+        hs[j] = a.gh[0];
+#pragma unroll
+        for (int g = 1; g < FF_MAX_GROUPS; ++g)
+            if (g < a.n_groups && i >= a.gstart[g]) hs[j] = a.gh[g];
+    }
+    const float pva = PP ? a.pparam[i0] : 0.0f, pvb = PP ? a.pparam[i0 + PER - 1] : 0.0f;
+#pragma unroll
+    for (int q = 0; q < HH3::NP; ++q) {
+        pa[q] = (PP && q == a.pidx) ? pva : a.p[q];
+        pb[q] = (PP && q == a.pidx) ? pvb : a.p[q];
+    }
+}
+
 template <bool PP, bool TAPE>
 __device__ __forceinline__ void hh3_rk4_x2_item(const IntegrateArgs& a, int64_t t, int n_steps) {
     constexpr int D = HH3::DIM;
@@ -1375,20 +1395,7 @@ __device__ __forceinline__ void hh3_rk4_x2_item(const IntegrateArgs& a, int64_t 
         X[k] = pack2(v[0], v[1]);
     }
     float hs[2], pa[HH3::NP], pb[HH3::NP];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const int64_t i = i0 + j;
-        hs[j] = a.gh[0];
-#pragma unroll
-        for (int g = 1; g < FF_MAX_GROUPS; ++g)
-            if (g < a.n_groups && i >= a.gstart[g]) hs[j] = a.gh[g];
-    }
-    const float pva = PP ? a.pparam[i0] : 0.0f, pvb = PP ? a.pparam[i0 + 1] : 0.0f;
-#pragma unroll
-    for (int q = 0; q < HH3::NP; ++q) {
-        pa[q] = (PP && q == a.pidx) ? pva : a.p[q];
-        pb[q] = (PP && q == a.pidx) ? pvb : a.p[q];
-    }
+    hh_pair_params<PP>(a, i0, hs, pa, pb);
     const HHConst<HHPair> c = hh_const_pair(pa, pb);
     f2 drive[3];
 #pragma unroll
@@ -1400,10 +1407,7 @@ __device__ __forceinline__ void hh3_rk4_x2_item(const IntegrateArgs& a, int64_t 
     auto step = [&]() {
         f2 XS[D], A[D];
 #pragma unroll
-        for (int k = 0; k < D; ++k) {
-            XS[k] = X[k];
-            A[k] = pack2(0.0f, 0.0f);
-        }
+        for (int k = 0; k < D; ++k) XS[k] = X[k];
         // the stages unrolled: 4% faster than a stage loop on hh3_1M (168 registers)
 #pragma unroll
         for (int st = 0; st < 4; ++st) {
@@ -1417,10 +1421,8 @@ __device__ __forceinline__ void hh3_rk4_x2_item(const IntegrateArgs& a, int64_t 
 #pragma unroll
                 for (int k = 0; k < 5; ++k) K[5 * n + k] = d[k];
             }
-            const float w = (st == 1 || st == 2) ? 2.0f : 1.0f;  // fmaf(1, k, 0) = k
-            const f2 W = pack2(w, w);
 #pragma unroll
-            for (int k = 0; k < D; ++k) A[k] = fma2(W, K[k], A[k]);
+            for (int k = 0; k < D; ++k) A[k] = rk4_weigh<HHPair>(st, K[k], A[k]);
             if (st == 3) break;
             const f2 C = (st == 2) ? H1 : H2;
 #pragma unroll
@@ -1444,26 +1446,6 @@ __device__ __forceinline__ void hh3_rk4_x2_item(const IntegrateArgs& a, int64_t 
         float v[2];
         unpack2(X[k], v[0], v[1]);
         Vec<2>::store(a.x + k * a.pitch + i0, v);
-    }
-}
-
-// HH3::f with neurons 0 and 1 packed in f32x2 registers and neuron 2 on floats, as
-// in HH3RK4Packed: lane by lane the same operations as HH3::f, so the same bits.
-__device__ __forceinline__ void hh3_f_packed(const float (&x)[15], const float* p, float (&dx)[15]) {
-    const HHConst<HHPair> c2 = hh_const<HHPair>(p);
-    const HHConst<HHScalar> c1 = hh_const<HHScalar>(p);
-    const float s_sum = __fadd_rn(__fadd_rn(x[4], x[9]), x[14]);
-    f2 X[5], K[5];
-    float k2[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) X[k] = pack2(x[k], x[5 + k]);
-    hh_neuron<HHPair>(X[0], X[1], X[2], X[3], X[4], sub2(pack2(s_sum, s_sum), X[4]),
-                      pack2(hh_drive_c(p, 0), hh_drive_c(p, 1)), c2, K);
-    hh_neuron<HHScalar>(x[10], x[11], x[12], x[13], x[14], __fsub_rn(s_sum, x[14]), hh_drive_c(p, 2), c1, k2);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        unpack2(K[k], dx[k], dx[5 + k]);
-        dx[10 + k] = k2[k];
     }
 }
 

@@ -69,3 +69,37 @@ def test_seeding_is_the_double_formula_for_every_box(count):
         got = np.empty((2, count), np.float32)
         s.get_state(got)
         np.testing.assert_array_equal(got.view(np.uint32), want.view(np.uint32), err_msg=f"{a} {b}")
+
+
+HH = [1.0, 120.0, 36.0, 0.3, 50.0, -77.0, -54.4, 0.5, -80.0, 8.0, 12.0, 10.0, 0.1, 10.0, 0.5, -20.0]
+HH_BOX = ([-80.0, 0.0, 0.0, 0.0, 0.0] * 3, [40.0, 1.0, 1.0, 1.0, 1.0] * 3)
+
+
+# HH x 3 at two particles per thread picks its kernel by size: a partial, full and just
+# overfull warp of 10 and of 20 particles, and either side of the lines between kernels.
+@pytest.mark.parametrize("n", [1, 3, 9, 10, 11, 21, -1, -2, -3, -4, -5, -6])
+@pytest.mark.parametrize("variant", ["plain", "parameter", "taped"])
+def test_hh3_kernels_by_size_give_the_one_particle_bits(n, variant):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = {-1: 120 * sms, -2: 120 * sms + 1, -3: 400 * sms, -4: 400 * sms + 1, -5: 256 * sms, -6: 256 * sms + 1}.get(n, n)
+    out = []
+    for ppt in (1, 2):
+        s = ff.System("hh3", HH, n, stream=_stream())
+        back = n // 3  # a group boundary inside a pair where it is odd
+        s.seed(n - back, *HH_BOX, +1, 5)
+        if back:
+            s.seed(back, *HH_BOX, -1, 6)
+        s.set_launch(ppt)
+        if variant == "parameter":
+            s.set_particle_param(9, 5.0, 15.0)
+        if variant == "taped":
+            s.tape_begin(3, 8)
+        s.step(7, 0.01)
+        x = np.empty((15, n), np.float32)
+        s.get_state(x)
+        out.append(x)
+        if variant == "taped":
+            lam = torch.ones((15, n), device="cuda")
+            s.backward(lam, lam, 16)
+            out[-1] = np.concatenate([x, lam.cpu().numpy()])
+    np.testing.assert_array_equal(out[0], out[1])
