@@ -196,8 +196,9 @@ ff_status ff_get_particle_param(ff_system* sys, float* dst, int dst_is_device, i
  *   bound_lo/bound_hi: dim values each (rounded to float), or both NULL for no
  *   bounds; t_max <= 0: no age limit; check_every >= 1 enables the reset,
  *   0 disables it.  Ages and reset counts start at 0 and are cleared by ff_reset
- *   and ff_set_state.  Resetting particles run the scalar integrator (one
- *   particle per thread).
+ *   and ff_set_state.  Resetting particles run one particle per thread,
+ *   or with the same bits (RK4 on WILSON_COWAN and LORENZ, uncompensated, no
+ *   per-particle parameter, groups that start on even particles) two.
  * Errors: FF_ERR_INVALID_ARG for check_every < 0, only one of the bounds
  * given, non-finite or inverted bounds, non-finite t_max; FF_ERR_OOM. */
 ff_status ff_set_reset(ff_system* sys, const double* bound_lo, const double* bound_hi, double t_max,

@@ -1032,6 +1032,7 @@ LaunchRecord& last_launch_record() {
 
 cudaError_t launch_integrate(int rhs_id, int method, bool kahan, bool pp, const IntegrateArgs& a,
                              const LaunchShape& shape, cudaStream_t stream) {
+    if (reset_pairs(rhs_id, method, kahan, pp, a)) return launch_reset_pairs(rhs_id, a, shape, stream);
     switch (rhs_id) {
     case FF_RHS_LORENZ:
         if (kahan && lorenz_kahan_packed(method, pp, a, shape)) return launch_integrate_lorenz_kahan(pp, a, shape, stream);

@@ -1074,6 +1074,9 @@ cudaError_t launch_integrate_lorenz_kahan(bool pp, const IntegrateArgs& a, const
                                           cudaStream_t stream);
 cudaError_t launch_integrate_wc(int method, bool kahan, bool pp, const IntegrateArgs& a,
                                 const LaunchShape& shape, cudaStream_t stream);
+// Wilson-Cowan and Lorenz with particle reset as packed pairs (ff_integrate_reset.cu).
+bool reset_pairs(int rhs_id, int method, bool kahan, bool pp, const IntegrateArgs& a);
+cudaError_t launch_reset_pairs(int rhs_id, const IntegrateArgs& a, const LaunchShape& shape, cudaStream_t stream);
 cudaError_t launch_integrate_hh3(int method, bool kahan, bool pp, const IntegrateArgs& a,
                                  const LaunchShape& shape, cudaStream_t stream);
 cudaError_t launch_integrate_linear(int rhs_id, int method, bool kahan, bool pp,

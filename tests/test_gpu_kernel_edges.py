@@ -103,3 +103,48 @@ def test_hh3_kernels_by_size_give_the_one_particle_bits(n, variant):
             s.backward(lam, lam, 16)
             out[-1] = np.concatenate([x, lam.cpu().numpy()])
     np.testing.assert_array_equal(out[0], out[1])
+
+
+WC = [16.0, 12.0, 15.0, 3.0, 1.25, 0.0, 1.0, 1.0, 1.0, 4.0]
+
+
+def _states(s):
+    n, _, dim, _ = s.info()
+    x = np.empty((dim, n), np.float32)
+    s.get_state(x)
+    return x
+
+
+# Particle reset in packed pairs: single particles, odd and even totals and a second group,
+# against one-particle launches (an odd first group keeps those).
+@pytest.mark.parametrize("counts", [(1,), (2,), (1, 5), (64, 3), (4098, 2001), (4097, 2000)])
+@pytest.mark.parametrize("system", ["wilson_cowan", "lorenz"])
+@pytest.mark.parametrize("bounds,t_max,every", [(True, 0.0, 1), (False, 0.07, 1), (True, 0.11, 3)])
+def test_reset_pairs_match_particles_alone(counts, system, bounds, t_max, every):
+    """The same ensemble with each group's first particle cut off into a system of its own
+    (a slice, so it draws as itself): every state, age and count agrees bit for bit with the
+    ensemble cut after an even and after an odd particle, which swaps lanes and kernels."""
+    params, box, lim, dt = {
+        "wilson_cowan": (WC, ([0, 0], [1, 1]), ([0.1, 0.05], [0.9, 0.95]), 0.01),
+        "lorenz": ([10.0, 28.0, 8 / 3], ([-30, -30, 0], [30, 30, 60]), ([-20, -25, 2], [20, 25, 45]), 0.01)}[system]
+    dim = len(box[0])
+
+    def run(parts):
+        s = ff.System(system, params, sum(n for _, _, n, _ in parts), stream=_stream())
+        for g, first, n, total in parts:
+            s.seed_slice(n, first, total, *box, 1 if g == 0 else -1, 40 + g)
+        s.set_reset(*(lim if bounds else (None, None)), t_max, every)
+        s.step(13, dt)
+        s.step(20, dt)
+        x = _states(s)
+        age, res = (np.empty(x.shape[1], np.uint32) for _ in "ab")
+        s.get_reset_state(age, res)
+        return np.concatenate([x.view(np.uint32), age[None], res[None]])
+
+    whole = run([(g, 0, n, n) for g, n in enumerate(counts)])
+    start = 0
+    for g, n in enumerate(counts):
+        cut = min(n, 1 + 2 * (n // 5))  # odd: the second part's pairs are the whole's shifted by one
+        parts = [run([(g, 0, cut, n)])] + ([run([(g, cut, n - cut, n)])] if n > cut else [])
+        np.testing.assert_array_equal(np.concatenate(parts, axis=1), whole[:, start:start + n])
+        start += n
