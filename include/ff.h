@@ -331,8 +331,12 @@ ff_status ff_last_launch(ff_system* sys, char* kernel, int kernel_len, int* grid
  * compensated, then runs two particles per packed f32x2 instruction; HH3 takes
  * 1 or 2, and plain RK4 at 2 runs all three neurons of two particles packed,
  * bit-identical to 1, from 400 particles per SM on (smaller ensembles run one
- * neuron per thread, with the same bits); the default is 4 for RK4 on Lorenz, 2 when compensated,
- * 2 for plain RK4 on HH3, and 1 otherwise; 0 keeps the current value),
+ * neuron per thread, with the same bits); plain RK4 on WILSON_COWAN at 2 runs packed
+ * pairs, which round differently within the accuracy of single precision, for particles whose
+ * whole group (of which the system may hold a slice) has 650 particles per SM or more, untaped,
+ * without reset or per-particle parameter, and one particle per thread otherwise;
+ * the default is 4 for RK4 on Lorenz, 2 when compensated,
+ * 2 for plain RK4 on HH3 and WILSON_COWAN, and 1 otherwise; 0 keeps the current value),
  * threads per block (a multiple of 32 up to 1024, default 512 for RK4 on
  * Lorenz and 256 otherwise, 0 keeps the current value; clamped to the kernel's
  * maximum, 512 for the 2- and 3-dimensional systems and 256 for LINEAR and

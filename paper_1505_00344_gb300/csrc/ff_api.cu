@@ -141,7 +141,9 @@ ff_status ff_create_system(int rhs_id, int dim, const double* params, int n_para
     const bool packed_lorenz = rhs_id == FF_RHS_LORENZ && method == FF_RK4;
     // HH3 plain RK4: two particles per thread, all three neurons of the pair packed
     const bool packed_hh3 = rhs_id == FF_RHS_HH3 && method == FF_RK4 && !(flags & FF_FLAG_KAHAN);
-    s->ppt = packed_lorenz ? ((flags & FF_FLAG_KAHAN) ? 2 : 4) : (packed_hh3 ? 2 : 1);
+    // Wilson-Cowan plain RK4: pairs too, from the ensemble size on where they are ahead
+    const bool packed_wc = rhs_id == FF_RHS_WILSON_COWAN && method == FF_RK4 && !(flags & FF_FLAG_KAHAN);
+    s->ppt = packed_lorenz ? ((flags & FF_FLAG_KAHAN) ? 2 : 4) : (packed_hh3 || packed_wc ? 2 : 1);
     s->block = packed_lorenz ? 512 : 256;
     *out = s;
     return FF_OK;
@@ -484,8 +486,9 @@ static ff_status integrate_steps(ff_system* s, int64_t n_steps, double dt, const
                                  const TapePlan* tape = nullptr) {
     ff::IntegrateArgs a{};
     ff::fill_integrate_args(s, dt, &a);
-    const int ppt = s->ppt;
-    ff::LaunchShape shape{ppt, s->block, s->blocks_per_sm, s->num_sms};
+    ff::LaunchShape shape{s->ppt, s->block, s->blocks_per_sm, s->num_sms, s->tape_on};
+    for (int g = 0; g < s->n_groups; ++g)
+        if (s->groups[g].total >= ff::wide_group(s->num_sms)) shape.wide |= 1u << g;
     const bool kahan = (s->flags & FF_FLAG_KAHAN) != 0;
     const bool pp = s->pparam_index >= 0;
     if (s->check_every > 0) {

@@ -1058,7 +1058,12 @@ struct LaunchShape {
     int block;
     int blocks_per_sm;  // 0 = occupancy limit
     int num_sms;
+    bool taped = false;  // the steps are taped (with or without a checkpoint in this launch)
+    uint32_t wide = 0;   // groups whose whole group (a slice's too) has wide_group particles or more
 };
+
+// Size from which a whole group counts as wide (Wilson-Cowan's packed pairs are ahead).
+inline int64_t wide_group(int num_sms) { return 650 * (int64_t)num_sms; }
 
 cudaError_t launch_integrate(int rhs_id, int method, bool kahan, bool pp, const IntegrateArgs& a,
                              const LaunchShape& shape, cudaStream_t stream);
@@ -1170,9 +1175,9 @@ inline cudaError_t launch_reset_variants(int method, bool kahan, bool pp, const 
 
 // Deal the persistent grid's blocks out to the groups in proportion to their
 // sizes (at least one block per group) and launch the group-uniform kernel.
-template <class Kernel>
+template <class Kernel, class... More>
 inline cudaError_t uniform_launch(Kernel kernel, const IntegrateArgs& a0, const LaunchShape& s0,
-                                  cudaStream_t stream) {
+                                  cudaStream_t stream, More... more) {
     LaunchShape s = s0;
     cudaFuncAttributes attr;
     cudaError_t e = cudaFuncGetAttributes(&attr, kernel);
@@ -1181,7 +1186,7 @@ inline cudaError_t uniform_launch(Kernel kernel, const IntegrateArgs& a0, const 
     IntegrateArgs a = a0;
     const int ppt = s.ppt;
     int64_t items_all = 0;
-    for (int g = 0; g < a.n_groups; ++g) items_all += (a.gend[g] - a.gstart[g]) / ppt;
+    for (int g = 0; g < a.n_groups; ++g) items_all += (a.gend[g] - a.gstart[g] + ppt - 1) / ppt;
     s.block = spread_block(s.block, items_all, s.num_sms);
     int occ = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, s.block, 0);
@@ -1191,7 +1196,7 @@ inline cudaError_t uniform_launch(Kernel kernel, const IntegrateArgs& a0, const 
     const int64_t total = (int64_t)per_sm * s.num_sms;
     int next = 0;
     for (int g = 0; g < a.n_groups; ++g) {
-        const int64_t items = (a.gend[g] - a.gstart[g]) / ppt;
+        const int64_t items = (a.gend[g] - a.gstart[g] + ppt - 1) / ppt;
         int64_t nb = items_all > 0 ? (total * items + items_all / 2) / items_all : 1;
         const int64_t need = (items + s.block - 1) / s.block;
         if (nb > need) nb = need;
@@ -1200,7 +1205,7 @@ inline cudaError_t uniform_launch(Kernel kernel, const IntegrateArgs& a0, const 
         next += (int)nb;
     }
     a.gblk[a.n_groups] = next;
-    kernel<<<next, s.block, 0, stream>>>(a);
+    kernel<<<next, s.block, 0, stream>>>(a, more...);
     last_launch_record() = LaunchRecord{(const void*)kernel, next, s.block};
     return cudaGetLastError();
 }

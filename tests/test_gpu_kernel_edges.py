@@ -108,11 +108,89 @@ def test_hh3_kernels_by_size_give_the_one_particle_bits(n, variant):
 WC = [16.0, 12.0, 15.0, 3.0, 1.25, 0.0, 1.0, 1.0, 1.0, 4.0]
 
 
+def _wc(n, back, ppt, seed=11, first=None, total=None):
+    s = ff.System("wilson_cowan", WC, n, stream=_stream())
+    if total is None:
+        s.seed(n - back, [0, 0], [1, 1], +1, seed)
+        if back:
+            s.seed(back, [0, 0], [1, 1], -1, seed + 1)
+    else:
+        s.seed_slice(n, first, total, [0, 0], [1, 1], +1, seed)
+    s.set_launch(ppt)
+    return s
+
+
 def _states(s):
     n, _, dim, _ = s.info()
     x = np.empty((dim, n), np.float32)
     s.get_state(x)
     return x
+
+
+# Wilson-Cowan at two particles per thread: either side of the line between its kernels, odd
+# counts, a second group that starts inside a pair, a small group beside a large one.
+@pytest.mark.parametrize("extra,back,kernel", [(0, 0, "wc_rk4_x2u"), (-1, 0, "integrate_kernel"), (1000, 1000, "wc_rk4_x2u"),
+                                               (1002, 1001, "wc_rk4_x2u"), (1, 1, "wc_rk4_x2u"), (500, 1000, "integrate_kernel")])
+def test_wilson_cowan_pairs_by_size(extra, back, kernel):
+    """The packed pairs against an FP64 RK4: each step rounds a state below 1.5 (1.5 backward)
+    by at most an ulp or two of it and the errors grow with the map, at most e^3.2 (the largest
+    eigenvalue of the reversed flow, 3.2, over one time unit) backward: 100 steps stay within
+    1e-5 of max(|x|, 1), the package's bar for this system."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 650 * sms + extra
+    s = _wc(n, back, 0)
+    x = torch.from_numpy(_states(s)).cuda().double()
+    h = torch.full((n,), 0.01, dtype=torch.float64, device="cuda")
+    h[n - back:] *= -1.0 if back else 1.0
+    s.step(100, 0.01)
+    assert kernel in s.last_launch()["kernel"]
+
+    def f(E, I):
+        S = lambda a: 1.0 / (1.0 + torch.exp(-WC[8] * (a - WC[9])))  # noqa: E731
+        return torch.stack([-E + S(WC[0] * E - WC[1] * I + WC[4]), -I + S(WC[2] * E - WC[3] * I + WC[5])])
+
+    for _ in range(100):
+        k1 = f(*x)
+        k2 = f(*(x + 0.5 * h * k1))
+        k3 = f(*(x + 0.5 * h * k2))
+        k4 = f(*(x + h * k3))
+        x = x + h / 6 * (k1 + 2 * k2 + 2 * k3 + k4)
+    want = x.cpu().numpy()
+    assert (np.abs(_states(s) - want) / np.maximum(np.abs(want), 1.0)).max() <= 1e-5
+
+
+def test_wilson_cowan_slices_and_odd_values_match_the_whole():
+    """A slice of an ensemble takes its whole ensemble's kernel: the slices' states are the
+    whole's to the bit.  Infinite and NaN states give the one-particle kernel's."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 650 * sms
+    whole = _wc(n, 0, 0, first=0, total=n)
+    whole.step(50, 0.01)
+    for a, b in ((0, 10), (10, 4001), (4001, n)):
+        part = _wc(b - a, 0, 0, first=a, total=n)
+        part.step(50, 0.01)
+        np.testing.assert_array_equal(_states(part), _states(whole)[:, a:b])
+    # pieces beside each other that start and end inside a pair, and beside a small group
+    part = ff.System("wilson_cowan", WC, 17, stream=_stream())
+    part.seed_slice(5, 0, n, [0, 0], [1, 1], +1, 11)
+    part.seed(7, [0, 0], [1, 1], +1, 12)
+    part.seed_slice(5, 5, n, [0, 0], [1, 1], +1, 11)
+    part.step(50, 0.01)
+    got = _states(part)
+    np.testing.assert_array_equal(np.concatenate([got[:, :5], got[:, 12:]], axis=1), _states(whole)[:, :10])
+    small = _wc(7, 0, 1, seed=12)
+    small.step(50, 0.01)
+    np.testing.assert_array_equal(got[:, 5:12], _states(small))
+    odd = np.array([np.nan, np.inf, -np.inf, 3e38, -3e38, 1e30, 0.0, 1.0], np.float32)
+    x0 = np.tile(np.array(np.meshgrid(odd, odd)).reshape(2, -1), n // 64 + 1)[:, :n].copy()
+    got = []
+    for ppt in (1, 2):
+        s = _wc(n, 0, ppt)
+        s.set_state(x0)
+        s.step(3, 0.01)
+        got.append(_states(s))
+    np.testing.assert_array_equal(np.isfinite(got[0]), np.isfinite(got[1]))
+    np.testing.assert_array_equal(np.isnan(got[0]), np.isnan(got[1]))
 
 
 # Particle reset in packed pairs: single particles, odd and even totals and a second group,
