@@ -20,7 +20,7 @@
 // from last to first, each on stage points that cp.async copies brought into the
 // lane's shared-memory column while the step before ran, and apply the four
 // vector-Jacobian products, hand-differentiated from Eq. 6-11.
-// The parameter gradient is carried in thirteen FP32 sums per neuron and particle
+// The parameter gradient is carried in twelve FP32 sums per neuron and particle
 // over the chunk, from which the sixteen components are formed in FP64 at the
 // chunk's end (each a sum times a parameter constant); the FP64 sums are reduced
 // over particles through per-block partials in a fixed order.
@@ -126,9 +126,10 @@ __device__ __forceinline__ void lane_fwd(f2 (&X)[5], const LaneC& L, int src0, u
 }
 
 // FP32 sums over a chunk of one neuron lane's parameter contributions (v_V the
-// adjoint of V, w_s = v_s (1 - s) / tau_r, a1 = act (1 - act), act the synaptic
-// sigmoid), each with the factor that makes it a gradient component:
-enum { A_U, A_CUR, A_NA, A_NAE, A_K, A_KE, A_L, A_SYN, A_SYNE, A_TR, A_TD, A_SG, A_TH, A_N };
+// adjoint of V, w = v_s (1 - s), act the synaptic sigmoid), each with the factor that
+// makes it a gradient component.  The sum of dV/dt v_V, which 1/C's derivative needs, is
+// the currents' own sums times their conductances, formed at the chunk's end.
+enum { A_U, A_NA, A_NAE, A_K, A_KE, A_L, A_SYN, A_SYNE, A_TR, A_TD, A_SG, A_TH, A_N };
 struct LaneAcc {
     f2 r[A_N];
     __device__ __forceinline__ f2 get(int i) const { return r[i]; }
@@ -140,85 +141,96 @@ struct LaneAcc {
     __device__ __forceinline__ void fma(int i, f2 a, f2 b) { r[i] = fma2(a, b, r[i]); }
 };
 
+// The rates of the products.  The forward's bits are fixed by its own operations (hh_neuron);
+// the products only need the rates at its stage points, so they take the cheaper of two
+// equally accurate forms: one exponential per rate instead of a power chain over one, and one
+// reciprocal per denominator instead of shared ones, on a unit that is 12% busy here where the
+// FP32 pipe is the bound.  alpha_h = 0.07 e^(-(V+65)/20) = 2^(kA V + kA0), beta_n = 0.125
+// e^(-(V+65)/80) = 2^(kQ V + kQ0), beta_m = 4 e^(-(V+65)/18) = 2^(kB V + kB0), each factor folded
+// into its exponent; with e^(-(V+65)/10) = (alpha_h / 0.07)^2, the e^-ym, e^-yn and
+// e^(-(V+35)/10) of the other rates are e^2.5, e and e^3 over 0.0049 times alpha_h^2.  Each slope
+// and offset is the pair of neighbouring floats, and each of the last three factors the float,
+// whose error over -82..45 mV is smallest; the rates' rms errors there are 0.4 to 1.1 times the
+// forward's, and 2 times for beta_n (8e-8).
+constexpr float kA = -0.07213474810123444f, kA0 = -8.525259971618652f;
+constexpr float kQ = -0.01803368702530861f, kQ0 = -4.172189712524414f;
+constexpr float kB = -0.08014972507953644f, kB0 = -3.2097320556640625f;
+constexpr float kE25 = 2486.223388671875f, kE1 = 554.75146484375f, kE3 = 4099.08935546875f;
+
+// g(y) = y / (1 - e^-y) = 1 + y/2 + y^2/12 - ... and g'(y) = 1/2 + y/6 - y^3/180 + ... for |y| < 0.5,
+// the terms beyond y^4 and y^5 folded into the coefficients by minimax fits over the band
+// (largest errors 2.0e-8 and 8e-10).
+__device__ __forceinline__ void bernoulli_band(f2 y, f2& g, f2& dg) {
+    const f2 y2 = mulp(y, y);
+    g = fma2(kp(0.5f), y, fma2(y2, fma2(y2, kp(-0.00137746f), kp(0.08333245f)), kp(1.0f)));
+    dg = fma2(y, fma2(y2, fma2(y2, kp(0.00019555f), kp(-0.0055552f)), kp(1.0f / 6.0f)), kp(0.5f));
+}
+
 // One neuron lane's vector-Jacobian product at state x (others: the other two
 // neurons' s), for input v = (v_V, v_m, v_h, v_n, v_s) of its components:
-//   jx_V = sum over gates y of v_y (a_y' (1 - y) - b_y' y) + sigma a1 w_s - v_V g_tot / C
+//   jx_V = sum over gates y of v_y (a_y' (1 - y) - b_y' y) + sigma act (1 - act) w / tau_r - v_V g_tot / C
 //   jx_y = (d I / d y) v_V / C - v_y (a_y + b_y)        for y = m, h, n
-//   self = -v_s (act / tau_r + 1 / tau_d)                the own-s part of jx_s
+//   decay = act / tau_r + 1 / tau_d                     minus the own-s derivative of ds/dt
 //   syn  = g_syn (E_syn - V) v_V / C                      added to the other neurons' jx_s
-// with the rates of the forward right-hand side, and the parameter sums added to acc.
+// and the parameter sums added to acc.
 __device__ __forceinline__ void lane_vjp(const f2 (&x)[5], f2 others, const f2 (&v)[5], const LaneC& L, f2 (&jx)[4],
-                                         f2& self, f2& syn, LaneAcc& acc) {
+                                         f2& decay, f2& syn, LaneAcc& acc) {
     using O = HHPair;
-    constexpr float kE25 = 12.182493960703473f;  // e^2.5
-    constexpr float kE1 = 2.718281828459045f;    // e^1
-    constexpr float kE3 = 20.085536923187668f;   // e^3
-    constexpr float kQ = -kLog2e / 80.0f, kQ0 = 65.0f * (-kLog2e / 80.0f);
-    constexpr float kB = -kLog2e / 18.0f, kB0 = 65.0f * (-kLog2e / 18.0f) + 2.0f;
     const f2 V = x[0], m = x[1], h = x[2], n = x[3], s = x[4];
     const f2 one = kp(1.0f);
     // rates and their derivatives
-    const f2 q = O::ex2(fma2(V, kp(kQ), kp(kQ0)));
-    const f2 q2 = mulp(q, q), q4 = mulp(q2, q2), q8 = mulp(q4, q4);
+    const f2 ah = O::ex2(fma2(V, kp(kA), kp(kA0)));
+    const f2 bn = O::ex2(fma2(V, kp(kQ), kp(kQ0)));
     const f2 bm = O::ex2(fma2(V, kp(kB), kp(kB0)));
-    const f2 ah = mulp(kp(0.07f), q4);
-    const f2 bn = mulp(kp(0.125f), q);
     const f2 es = O::ex2(fma2(L.c.neg_sig2, V, L.c.sig2_theta));
+    const f2 ah2 = mulp(ah, ah);
     const f2 ym = fma2(V, kp(0.1f), kp(4.0f)), yn = fma2(V, kp(0.1f), kp(5.5f));
     const auto sm = O::small(ym), sn = O::small(yn);
-    const f2 em = mulp(kp(kE25), q8), en = mulp(kp(kE1), q8);
-    const f2 dm = O::sel(sm, one, sub2(one, em)), dn = O::sel(sn, one, sub2(one, en));
-    const f2 rmn = O::rcp(mulp(dm, dn));
-    const f2 rm = mulp(dn, rmn), rn = mulp(dm, rmn);  // 1 / dm, 1 / dn
+    const f2 em = mulp(kp(kE25), ah2), en = mulp(kp(kE1), ah2);
+    const f2 rm = O::rcp(sub2(one, em)), rn = O::rcp(sub2(one, en));
     // g(y) = y r with r = 1 / (1 - e^-y), and g'(y) = (1 - e^-y - y e^-y) r^2 = r (1 - e^-y g);
     // alpha_m = g(ym), alpha_n = g(yn) / 10; at most one of ym, yn lies in the series band
-    const f2 ys = O::sel(sm, ym, yn);
-    const f2 ser = bernoulli_series_t<O>(ys), dser = bernoulli_series_deriv_t<O>(ys);
+    f2 ser, dser;
+    bernoulli_band(O::sel(sm, ym, yn), ser, dser);
     const f2 gmc = mulp(ym, rm), gnc = mulp(yn, rn);  // the closed forms
     const f2 am = O::sel(sm, ser, gmc);
     const f2 gn = O::sel(sn, ser, gnc);
     const f2 dgm = O::sel(sm, dser, mulp(O::fms(em, gmc, one), rm));
     const f2 dgn = O::sel(sn, dser, mulp(O::fms(en, gnc, one), rn));
     const f2 anbn = fma2(kp(0.1f), gn, bn);
-    const f2 dam = mulp(kp(0.1f), dgm), dan = mulp(kp(0.01f), dgn);
-    const f2 ph = fma2(kp(kE3), q8, one), ps = add2(one, es);
-    const f2 r = O::rcp(mulp(ph, ps));
-    const f2 bh = mulp(ps, r), act = mulp(ph, r);
-    const f2 a1 = mulp(act, sub2(one, act));
-    // minus the beta derivatives: beta_m' = -beta_m/18, beta_n' = -beta_n/80, beta_h' = beta_h (1 - beta_h)/10
-    const f2 nd_bm = mulp(bm, kp(1.0f / 18.0f)), nd_bn = mulp(bn, kp(1.0f / 80.0f));
-    const f2 nd_bh = mulp(mulp(kp(0.1f), bh), sub2(bh, one));
-    const f2 dah = mulp(ah, kp(-1.0f / 20.0f));
-    // currents and conductances, divided by C
-    const f2 m2 = mulp(m, m), m3 = mulp(m2, m), m3h = mulp(m3, h);
-    const f2 n2 = mulp(n, n), n3 = mulp(n2, n), n4 = mulp(n2, n2);
-    const f2 dNa = sub2(L.c.ENa, V), dK = sub2(L.c.EK, V), dL = sub2(L.c.EL, V), dS = sub2(L.c.Esyn, V);
-    const f2 gna = mulp(L.c.gNaC, m3h), gk = mulp(L.c.gKC, n4), gs = mulp(L.c.gsynC, others);
-    f2 I = fma2(L.c.gLC, dL, L.driveC);
-    I = fma2(gna, dNa, I);
-    I = fma2(gk, dK, I);
-    I = fma2(gs, dS, I);
-    const f2 gtot = add2(gs, add2(gk, add2(gna, L.c.gLC)));
+    const f2 bh = O::rcp(fma2(kp(kE3), ah2, one));
+    const f2 act = O::rcp(add2(one, es)), actr = mulp(act, L.c.inv_tr);
     // state
     const f2 vV = v[0];
-    const f2 ws = mulp(mulp(v[4], L.c.inv_tr), sub2(one, s));  // v_s (1 - s) / tau_r
-    // a' (1 - y) - b' y = a' + y (-b' - a')
-    const f2 gate_m = fma2(m, sub2(nd_bm, dam), dam);
-    const f2 gate_h = fma2(h, sub2(nd_bh, dah), dah);
-    const f2 gate_n = fma2(n, sub2(nd_bn, dan), dan);
-    const f2 a1ws = mulp(a1, ws);
-    const f2 jv = fma2(v[1], gate_m, fma2(v[2], gate_h, fma2(v[3], gate_n, mulp(L.sig, a1ws))));
-    jx[0] = O::fms(vV, gtot, jv);
-    const f2 wNa = mulp(vV, dNa);
-    jx[1] = O::fms(v[1], add2(am, bm), mulp(mulp(mulp(L.gNa3C, m2), h), wNa));
-    jx[2] = O::fms(v[2], add2(ah, bh), mulp(mulp(L.c.gNaC, m3), wNa));
+    const f2 aw = mulp(actr, mulp(v[4], sub2(one, s)));  // act w / tau_r
+    const f2 a1w = mulp(aw, sub2(one, act));             // act (1 - act) w / tau_r
+    // minus a' (1 - y) - b' y, as -a' - y (-b' - a'), with beta_m' = -beta_m/18, beta_n' =
+    // -beta_n/80, beta_h' = beta_h (1 - beta_h)/10 and alpha_h' = -alpha_h/20
+    const f2 ndam = mulp(kp(-0.1f), dgm), ndan = mulp(kp(-0.01f), dgn), ndah = mulp(kp(1.0f / 20.0f), ah);
+    const f2 ngate_m = O::fms(m, fma2(kp(1.0f / 18.0f), bm, ndam), ndam);
+    const f2 ngate_h = O::fms(h, fma2(mulp(kp(0.1f), bh), sub2(bh, one), ndah), ndah);
+    const f2 ngate_n = O::fms(n, fma2(kp(1.0f / 80.0f), bn, ndan), ndan);
+    f2 jv = mulp(L.sig, a1w);
+    jv = O::fms(v[3], ngate_n, jv);
+    jv = O::fms(v[2], ngate_h, jv);
+    jv = O::fms(v[1], ngate_m, jv);
+    // currents: each conductance's part of -v_V g_tot / C from its parameter sum's term
+    const f2 m2 = mulp(m, m), m3 = mulp(m2, m);
+    const f2 n2 = mulp(n, n), n3 = mulp(n2, n), n4 = mulp(n2, n2);
+    const f2 dNa = sub2(L.c.ENa, V), dK = sub2(L.c.EK, V), dL = sub2(L.c.EL, V), dS = sub2(L.c.Esyn, V);
+    const f2 tna = mulp(mulp(m3, h), vV), tk = mulp(n4, vV), ts = mulp(others, vV);
+    jv = O::fms(L.c.gLC, vV, jv);
+    jv = O::fms(L.c.gsynC, ts, jv);
+    jv = O::fms(L.c.gKC, tk, jv);
+    jx[0] = O::fms(L.c.gNaC, tna, jv);
+    const f2 wNa = mulp(m2, mulp(vV, dNa));
+    jx[1] = O::fms(v[1], add2(am, bm), mulp(mulp(L.gNa3C, h), wNa));
+    jx[2] = O::fms(v[2], add2(ah, bh), mulp(mulp(L.c.gNaC, m), wNa));
     jx[3] = O::fms(v[3], anbn, mulp(mulp(mulp(L.gK4C, n3), dK), vV));
-    self = mulp(v[4], O::fms(act, L.c.inv_tr, L.c.neg_inv_td));  // -v_s (act / tau_r + 1 / tau_d)
+    decay = sub2(actr, L.c.neg_inv_td);
     syn = mulp(mulp(L.c.gsynC, dS), vV);
     // parameter sums
     acc.add(A_U, vV);
-    acc.fma(A_CUR, I, vV);
-    const f2 tna = mulp(m3h, vV), tk = mulp(n4, vV), ts = mulp(others, vV);
     acc.add(A_NAE, tna);
     acc.fma(A_NA, tna, dNa);
     acc.add(A_KE, tk);
@@ -226,22 +238,22 @@ __device__ __forceinline__ void lane_vjp(const f2 (&x)[5], f2 others, const f2 (
     acc.fma(A_L, dL, vV);
     acc.add(A_SYNE, ts);
     acc.fma(A_SYN, ts, dS);
-    acc.fma(A_TR, act, ws);
+    acc.add(A_TR, aw);
     acc.fma(A_TD, s, v[4]);
-    acc.add(A_TH, a1ws);
-    acc.fma(A_SG, a1ws, V);
+    acc.add(A_TH, a1w);
+    acc.fma(A_SG, a1w, V);
 }
 
 // The product at stage point x (others from the triple's s sum at it) and the full
-// adjoint of the lane's components: jx_s gains the other two neurons' synaptic terms,
-// (syn0 + syn1) + syn2 - syn_own.
+// adjoint of the lane's components: jx_s is -v_s decay plus the other two neurons'
+// synaptic terms, (syn0 + syn1) + syn2 - syn_own.
 __device__ __forceinline__ void lane_product(const f2 (&x)[5], f2 s_sum, const f2 (&v)[5], const LaneC& L, f2 (&out)[5],
                                              LaneAcc& acc, int src0) {
-    f2 jx[4], self, syn;
-    lane_vjp(x, sub2(s_sum, x[4]), v, L, jx, self, syn, acc);
+    f2 jx[4], decay, syn;
+    lane_vjp(x, sub2(s_sum, x[4]), v, L, jx, decay, syn, acc);
 #pragma unroll
     for (int k = 0; k < 4; ++k) out[k] = jx[k];
-    out[4] = add2(self, sub2(triple_sum(syn, src0), syn));
+    out[4] = HHPair::fms(v[4], decay, sub2(triple_sum(syn, src0), syn));
 }
 
 // Reverse of one RK4 step of the lane's neuron, from its stage points x1 = x,
@@ -310,12 +322,14 @@ __device__ __forceinline__ float group_h(const AdjointArgs& a, const AdjChunk& c
 
 // The sixteen parameter components of one particle's chunk sums (one lane of each
 // register of acc), added to gacc (FP64).
-__device__ __forceinline__ void add_chunk_grads(const float (&p)[HH3::NP], int n, float u, float cur, float na,
-                                                float na_e, float k, float k_e, float l, float syn, float syn_e,
-                                                float tr, float td, float sg, float th, double* gacc, int bs) {
+__device__ __forceinline__ void add_chunk_grads(const float (&p)[HH3::NP], int n, float u, float na, float na_e,
+                                                float k, float k_e, float l, float syn, float syn_e, float tr,
+                                                float td, float sg, float th, double* gacc, int bs) {
     const double invC = 1.0 / (double)p[0], inv_tr = 1.0 / (double)p[12], inv_td = 1.0 / (double)p[13];
     double g[HH3::NP];
-    g[0] = -(double)cur * invC;
+    const double cur = (double)p[9 + n] * u + (double)p[1] * na + (double)p[2] * k + (double)p[3] * l +
+                       (double)p[7] * syn;  // C times the sum of dV/dt v_V
+    g[0] = -cur * invC * invC;
     g[1] = (double)na * invC;
     g[2] = (double)k * invC;
     g[3] = (double)l * invC;
@@ -412,9 +426,8 @@ __device__ __forceinline__ void lane_sweep(const AdjointArgs& a, int64_t first, 
                 lane_adj_rk4(stage + half * kStepPoints * bs, bs, lam, L, acc, src0);
             }
         }
-        float u[2], cur[2], na[2], na_e[2], kk[2], k_e[2], l[2], syn[2], syn_e[2], tr[2], td[2], sg[2], th[2];
+        float u[2], na[2], na_e[2], kk[2], k_e[2], l[2], syn[2], syn_e[2], tr[2], td[2], sg[2], th[2];
         unpack2(acc.get(A_U), u[0], u[1]);
-        unpack2(acc.get(A_CUR), cur[0], cur[1]);
         unpack2(acc.get(A_NA), na[0], na[1]);
         unpack2(acc.get(A_NAE), na_e[0], na_e[1]);
         unpack2(acc.get(A_K), kk[0], kk[1]);
@@ -431,7 +444,7 @@ __device__ __forceinline__ void lane_sweep(const AdjointArgs& a, int64_t first, 
             if (e == 0 ? !v0 : !v1) continue;
             float p[HH3::NP];
             lane_params<PP>(a, ch, e == 0 ? i0 : i1, p);
-            add_chunk_grads(p, n, u[e], cur[e], na[e], na_e[e], kk[e], k_e[e], l[e], syn[e], syn_e[e], tr[e], td[e],
+            add_chunk_grads(p, n, u[e], na[e], na_e[e], kk[e], k_e[e], l[e], syn[e], syn_e[e], tr[e], td[e],
                             sg[e], th[e], gacc, bs);
         }
     }

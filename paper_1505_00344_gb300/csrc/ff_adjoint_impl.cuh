@@ -88,14 +88,6 @@ template <> struct Vjp<WilsonCowan> {
     }
 };
 
-// d/dy of y / (1 - e^-y) by its series 1/2 + y/6 - y^3/180 + y^5/5040 - y^7/151200 (|y| < 0.5).
-template <class O>
-__device__ __forceinline__ typename O::T bernoulli_series_deriv_t(typename O::T y) {
-    const auto y2 = O::mul(y, y);
-    return O::fma(y, O::fma(y2, O::fma(y2, O::fma(y2, O::k(-1.0f / 151200.0f), O::k(1.0f / 5040.0f)),
-                                       O::k(-1.0f / 180.0f)), O::k(1.0f / 6.0f)), O::k(0.5f));
-}
-
 template <> struct Vjp<Linear> {
     // f = A x (A padded to 8x8 row-major)
     __device__ __forceinline__ static void apply(const float (&x)[8], const float* p, const float (&v)[8],
