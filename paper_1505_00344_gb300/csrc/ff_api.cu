@@ -160,6 +160,7 @@ ff_status ff_destroy_system(ff_system* s) {
     cudaFree(s->d_stage);
     cudaFree(s->d_tiles);
     cudaFree(s->d_entries);
+    cudaFree(s->d_planes);
     cudaFree(s->d_age);
     cudaFree(s->d_resets);
     cudaFree(s->d_reset_table);
@@ -720,9 +721,9 @@ ff_status ff_backward(ff_system* s, const float* dL_dxT_dev, float* dL_dx0_dev, 
 
 // The device image a render call draws into: the caller's device image, or the
 // system's staging buffer holding (when accumulating) a copy of the caller's host
-// image; cleared first unless accumulating.
+// image; cleared first unless accumulating or (clear false) written whole by the caller.
 static ff_status image_begin(ff_system* s, void* image, int image_is_device, size_t bytes, int accumulate,
-                             void** target, const char* who) {
+                             void** target, const char* who, bool clear = true) {
     cudaError_t e = cudaSuccess;
     *target = image;
     if (!image_is_device) {
@@ -737,7 +738,7 @@ static ff_status image_begin(ff_system* s, void* image, int image_is_device, siz
         *target = s->d_stage;
         if (accumulate) e = cudaMemcpyAsync(*target, image, bytes, cudaMemcpyHostToDevice, s->stream);
     }
-    if (e == cudaSuccess && !accumulate) e = cudaMemsetAsync(*target, 0, bytes, s->stream);
+    if (e == cudaSuccess && !accumulate && clear) e = cudaMemsetAsync(*target, 0, bytes, s->stream);
     if (e != cudaSuccess) return cuda_fail(e, who);
     return FF_OK;
 }
@@ -865,17 +866,60 @@ ff_status ff_project_sprites(ff_system* s, const ff_view* v, const ff_sprite* sp
     const bool tiles_fit = n_tiles <= ff::kSpriteMaxTiles && entries < ((int64_t)1 << 31);
     if (sp->technique == FF_SPRITE_TILED && !tiles_fit)
         return fail(FF_ERR_UNSUPPORTED, "ff_project_sprites: %d tiles, more than the tiled technique takes", n_tiles);
-    // AUTO takes the direct technique: measured faster on every workload tried (the L2's
-    // vector reductions outrun shared-memory atomics on the dense tiles of an attractor)
     const bool tiled = sp->technique == FF_SPRITE_TILED;
+    // AUTO: weight planes where they save reductions enough, else one reduction per fragment
+    // (both ahead of the tiles on every workload tried: the L2's vector reductions outrun
+    // shared-memory atomics on the dense tiles of an attractor)
+    ff::SpritePlanes pl{};
+    for (int g = 0; g < FF_MAX_GROUPS; ++g) {
+        pl.slot[g] = -1;
+        if (g < s->n_groups && ((a.v.mask >> g) & 1u)) {
+            pl.colour[pl.n] = a.colour[g];
+            pl.slot[g] = pl.n++;
+        }
+    }
+    bool planes = sp->technique == FF_SPRITE_AUTO && s->n_particles > 0 &&
+                  ff::sprite_planes_pay(s->n_particles, pl.n, v->width, v->height, sp->radius);
 
     DeviceScope dev(s->device);
     if (dev.err != cudaSuccess) return cuda_fail(dev.err, "ff_project_sprites: set device");
     const size_t bytes = sizeof(float) * 4 * (size_t)v->width * v->height;
-    void* target = nullptr;
-    ff_status ist = image_begin(s, image, image_is_device, bytes, v->accumulate, &target, "ff_project_sprites");
-    if (ist != FF_OK) return ist;
     cudaError_t e = cudaSuccess;
+    if (planes) {
+        // under stream capture: the direct technique, which has no workspace to allocate or outlive
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        e = cudaStreamIsCapturing(s->stream, &cap);
+        if (e != cudaSuccess) return cuda_fail(e, "ff_project_sprites: capture status");
+        planes = cap == cudaStreamCaptureStatusNone;
+    }
+    if (planes && !s->planes_asked) {
+        // a system's first picture does not pay for the workspace (about 20 us to allocate and clear)
+        s->planes_asked = true;
+        planes = false;
+    }
+    if (planes) {
+        pl.wb = (v->width + 1) / 2;
+        pl.hb = (v->height + 1) / 2;
+        pl.stride = (int64_t)pl.wb * pl.hb;
+        const size_t need = (size_t)pl.stride * pl.n;
+        if (s->planes_cap < need) {
+            cudaFree(s->d_planes);
+            s->d_planes = nullptr;
+            s->planes_cap = 0;
+            if (cudaMalloc(&s->d_planes, sizeof(float4) * need) == cudaSuccess) {
+                s->planes_cap = need;
+                e = cudaMemsetAsync(s->d_planes, 0, sizeof(float4) * need, s->stream);
+                if (e != cudaSuccess) return cuda_fail(e, "ff_project_sprites: weight planes");
+            } else {
+                cudaGetLastError();  // no room: the direct technique needs none
+                planes = false;
+            }
+        }
+        pl.w = s->d_planes;
+    }
+    void* target = nullptr;
+    ff_status ist = image_begin(s, image, image_is_device, bytes, v->accumulate, &target, "ff_project_sprites", !planes);
+    if (ist != FF_OK) return ist;
     a.image = static_cast<float4*>(target);
     if (tiled) {
         const size_t need_tiles = 4 * (size_t)n_tiles + 2;
@@ -897,8 +941,9 @@ ff_status ff_project_sprites(ff_system* s, const ff_view* v, const ff_sprite* sp
         }
     }
     if (s->n_particles > 0 && a.v.mask != 0) {
-        e = tiled ? ff::launch_sprites_tiled(a, v->ndim_view, masked, s->d_tiles, s->d_entries, s->num_sms, s->stream)
-                  : ff::launch_sprites(a, v->ndim_view, masked, s->num_sms, s->stream);
+        e = planes  ? ff::launch_sprites_planes(a, pl, v->ndim_view, v->accumulate != 0, s->num_sms, s->stream)
+            : tiled ? ff::launch_sprites_tiled(a, v->ndim_view, masked, s->d_tiles, s->d_entries, s->num_sms, s->stream)
+                    : ff::launch_sprites(a, v->ndim_view, masked, s->num_sms, s->stream);
         if (e != cudaSuccess) return cuda_fail(e, "sprite kernel launch");
     }
     return image_end(s, image, image_is_device, bytes, target, "ff_project_sprites");

@@ -48,6 +48,21 @@ struct SpriteArgs {
     float4 colour[FF_MAX_GROUPS];  // gain * colour per group
 };
 
+// Sprites through weight planes: per drawn group one plane of summed weights, stored as 2 x 2
+// pixel blocks of 16 bytes, which a second kernel turns into the image.
+struct SpritePlanes {
+    float4* w;             // plane p, block (bx, by) at w[p * stride + by * wb + bx]; zero between calls
+    int64_t stride;        // blocks per plane
+    int wb, hb;            // blocks per row, rows of blocks
+    int n;                 // planes
+    int slot[FF_MAX_GROUPS];   // plane of each group, -1 if it is not drawn
+    float4 colour[FF_MAX_GROUPS];  // gain * colour of each plane
+};
+// Whether the planes are expected to be ahead of one reduction per fragment (see sprite_plane_kernel).
+bool sprite_planes_pay(int64_t n, int drawn_groups, int W, int H, float radius);
+cudaError_t launch_sprites_planes(const SpriteArgs& a, const SpritePlanes& p, int ndim_view, bool accumulate,
+                                  int num_sms, cudaStream_t s);
+
 cudaError_t launch_seed(const SeedArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_sprites(const SpriteArgs& a, int ndim_view, bool masked, int num_sms, cudaStream_t s);
 

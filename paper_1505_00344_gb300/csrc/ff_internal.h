@@ -78,6 +78,9 @@ struct ff_system {
     size_t tiles_cap = 0;  // uint32 entries
     uint32_t* d_entries = nullptr;
     size_t entries_cap = 0;
+    float4* d_planes = nullptr;  // sprite weight planes, zero between calls
+    size_t planes_cap = 0;       // 2 x 2 blocks
+    bool planes_asked = false;   // a picture has asked for them: the next one allocates them
     // launch shape
     int ppt = 1, block = 256, blocks_per_sm = 0;
     int64_t max_steps = 0;
