@@ -987,15 +987,34 @@ ff_status ff_step_splat(ff_system* s, int64_t n_steps, double dt, const ff_view*
     return FF_OK;
 }
 
+// Whether a caller's buffer is plain memory of the system's device, which a kernel may access
+// (not another device's, a mapped host buffer or an unaligned pointer: those take the copy call).
+static bool device_local(const ff_system* s, const void* p) {
+    if (reinterpret_cast<uintptr_t>(p) & 3u) return false;
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == s->device;
+}
+
+// dim planes of P floats between the system's state and a caller's [dim][P].
+static cudaError_t copy_state(ff_system* s, float* dst, int64_t dst_pitch, const float* src, int64_t src_pitch,
+                              const void* callers, cudaMemcpyKind kind) {
+    if (kind == cudaMemcpyDeviceToDevice && device_local(s, callers))
+        return ff::launch_copy_planes(dst, dst_pitch, src, src_pitch, s->n_particles, s->dim, s->num_sms, s->stream);
+    return cudaMemcpy2DAsync(dst, sizeof(float) * dst_pitch, src, sizeof(float) * src_pitch,
+                             sizeof(float) * s->n_particles, s->dim, kind, s->stream);
+}
+
 ff_status ff_get_state(ff_system* s, float* dst, int dst_is_device) {
     if (!s || !dst) return fail(FF_ERR_INVALID_ARG, "ff_get_state: NULL argument");
     DeviceScope dev(s->device);
     if (dev.err != cudaSuccess) return cuda_fail(dev.err, "ff_get_state: set device");
     if (s->n_particles == 0) return FF_OK;
-    cudaError_t e = cudaMemcpy2DAsync(dst, sizeof(float) * s->n_particles, s->d_state, sizeof(float) * s->pitch,
-                                      sizeof(float) * s->n_particles, s->dim,
-                                      dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                                      s->stream);
+    cudaError_t e = copy_state(s, dst, s->n_particles, s->d_state, s->pitch, dst,
+                               dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost);
     if (e == cudaSuccess && !dst_is_device) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_fail(e, "ff_get_state: copy");
     return FF_OK;
@@ -1006,10 +1025,8 @@ ff_status ff_set_state(ff_system* s, const float* src, int src_is_device) {
     if (s->n_particles < 1) return fail(FF_ERR_STATE, "ff_set_state: no particles seeded");
     DeviceScope dev(s->device);
     if (dev.err != cudaSuccess) return cuda_fail(dev.err, "ff_set_state: set device");
-    cudaError_t e = cudaMemcpy2DAsync(s->d_state, sizeof(float) * s->pitch, src, sizeof(float) * s->n_particles,
-                                      sizeof(float) * s->n_particles, s->dim,
-                                      src_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                                      s->stream);
+    cudaError_t e = copy_state(s, s->d_state, s->pitch, src, s->n_particles, src,
+                               src_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice);
     if (e == cudaSuccess && s->d_comp)
         e = cudaMemsetAsync(s->d_comp, 0, sizeof(float) * (size_t)s->pitch * s->dim, s->stream);
     if (e == cudaSuccess && !src_is_device) e = cudaStreamSynchronize(s->stream);

@@ -63,6 +63,10 @@ bool sprite_planes_pay(int64_t n, int drawn_groups, int W, int H, float radius);
 cudaError_t launch_sprites_planes(const SpriteArgs& a, const SpritePlanes& p, int ndim_view, bool accumulate,
                                   int num_sms, cudaStream_t s);
 
+// dim planes of n floats from src (src_pitch apart) to dst (dst_pitch apart), both in this device's
+// memory and aligned to 4 bytes.
+cudaError_t launch_copy_planes(float* dst, int64_t dst_pitch, const float* src, int64_t src_pitch, int64_t n, int dim,
+                               int num_sms, cudaStream_t s);
 cudaError_t launch_seed(const SeedArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_sprites(const SpriteArgs& a, int ndim_view, bool masked, int num_sms, cudaStream_t s);
 

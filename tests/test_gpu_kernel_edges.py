@@ -261,3 +261,26 @@ def test_sprite_planes_match_the_direct_technique(width, height, radius, mask, a
     assert (np.abs(out[0] - out[1]) <= bar).all()
     assert np.array_equal(out[0][out[1] == (base.cpu().numpy() if accumulate else 0)],
                           out[1][out[1] == (base.cpu().numpy() if accumulate else 0)])
+
+
+# Device copies of the state: runs of 4,096, planes at every offset modulo 16 bytes, an unaligned
+# base, a buffer the copy kernel may not touch (pinned host memory given by its address).
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 255, 4095, 4096, 4097, 8192, 12290])
+@pytest.mark.parametrize("dim,offset", [(2, 0), (3, 1), (15, 2), (15, 3)])
+def test_device_state_copies(n, dim, offset):
+    rhs, params = {2: ("harmonic", [1.0]), 3: ("lorenz", [10.0, 28.0, 8 / 3]), 15: ("hh3", HH)}[dim]
+    s = ff.System(rhs, params, n, stream=_stream())
+    s.seed(n, [0.0] * dim, [1.0] * dim, 1, 3)
+    want = _states(s)
+    buf = torch.full((dim * n + 8,), -7.0, device="cuda")
+    s.get_state(buf[offset:offset + dim * n])
+    got = buf.cpu().numpy()
+    np.testing.assert_array_equal(got[offset:offset + dim * n].reshape(dim, n), want)
+    assert (got[:offset] == -7).all() and (got[offset + dim * n:] == -7).all()
+    new = torch.rand(dim * n + 8, device="cuda")
+    s.set_state(new[offset:offset + dim * n])
+    np.testing.assert_array_equal(_states(s), new[offset:offset + dim * n].cpu().numpy().reshape(dim, n))
+    pinned = torch.zeros(dim * n).pin_memory()
+    ff.ff_get_state(s.handle, pinned.data_ptr())
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(pinned.numpy().reshape(dim, n), _states(s))
