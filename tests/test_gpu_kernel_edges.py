@@ -284,3 +284,29 @@ def test_device_state_copies(n, dim, offset):
     ff.ff_get_state(s.handle, pinned.data_ptr())
     torch.cuda.synchronize()
     np.testing.assert_array_equal(pinned.numpy().reshape(dim, n), _states(s))
+
+
+# Batch tiles by the batch's size: members of one particle and of odd counts, beside one large
+# enough that tiles grow to several items a thread, at the default and at tuned shapes.
+@pytest.mark.parametrize("counts", [(1, 2, 5), (63, 130, 4097), (7, 300_003, 900)])
+@pytest.mark.parametrize("tuned", [False, True])
+def test_batch_tiles_cover_every_particle(counts, tuned):
+    def members():
+        out = []
+        for q, n in enumerate(counts):
+            for name, p, box in (("hh3", HH, HH_BOX), ("wilson_cowan", WC, ([0, 0], [1, 1]))):
+                s = ff.System(name, p, n, stream=_stream())
+                s.seed(n, *box, +1, 50 + q)
+                out.append(s)
+        return out
+
+    batched, alone = members(), members()
+    dts = [0.01] * len(batched)
+    b = ff.Batch(batched, _stream())
+    if tuned:
+        b.autotune(dts, 2)
+    b.step(4, dts)
+    for x, y in zip(batched, alone):
+        y.set_launch(1)
+        y.step(4, 0.01)
+        np.testing.assert_array_equal(_states(x), _states(y))
