@@ -25,11 +25,11 @@
 namespace ff {
 
 // Column q of the partial rows [r0, r1), summed by one block in a fixed order: thread t adds
-// rows r0 + t, r0 + t + 128, ... and the threads' sums meet in a tree over lanes, then warps.
+// rows r0 + t, r0 + t + 512, ... and the threads' sums meet in a tree over lanes, then warps.
 // A chain of one dependent load and FP64 addition per row costs about 0.1 us each, which one
 // thread walking all rows paid 1,216 times on a 1M-particle Lorenz sweep (130 us, 4% of the
 // training step; 51 us of the 64k-particle HH x 3 one); split over a block both take 5-6 us.
-constexpr int kReduceBlock = 128;
+constexpr int kReduceBlock = 512;
 __device__ __forceinline__ void block_column_sum(const double* partial, int64_t r0, int64_t r1, int np_stride, int q,
                                                  double* out) {
     __shared__ double warp_sum[kReduceBlock / 32];
@@ -78,8 +78,10 @@ int64_t adjoint_scratch_threads(int rhs_id, int method, bool pp, int num_sms, bo
     return rhs_id == FF_RHS_HH3 ? adjoint_scratch_threads_hh3(method, pp, num_sms, batched) : 0;
 }
 
-cudaError_t launch_adjoint(int rhs_id, int method, bool pp, int m, const AdjointArgs& a, int num_sms,
+cudaError_t launch_adjoint(int rhs_id, int method, bool pp, int m, const AdjointArgs& a0, int num_sms,
                            cudaStream_t s, double* dL_dp_dev, int n_params_kernel) {
+    AdjointArgs a = a0;
+    if (adjoint_task_doubles(rhs_id, method, a.n) > 0) a.np_stride = kTaskRow;
     const int block = 128;
     int64_t rows = 0;
     cudaError_t e;

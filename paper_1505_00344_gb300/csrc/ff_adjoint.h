@@ -17,6 +17,8 @@ struct AdjChunk {
     float gh[FF_MAX_GROUPS];
 };
 
+struct WorkQueue;  // ff_device.cuh
+
 struct AdjointArgs {
     const float* ckpt;       // checkpoints, slot c at ckpt + c * dim * pitch (SoA planes)
     const AdjChunk* chunks;  // device table, in time order
@@ -34,6 +36,7 @@ struct AdjointArgs {
     int n_groups;
     int max_chunk;           // steps of the longest chunk (the tape's checkpoint spacing)
     int64_t gstart[FF_MAX_GROUPS];
+    WorkQueue* queue;         // packed Lorenz sweeps: hands out their warp tasks
     float* scratch;           // HH x 3 sweep: one chunk of stage points per thread (a neuron of two particles)
     int64_t scratch_threads;  // threads the scratch has room for (see adjoint_scratch_floats_per_step)
 };
@@ -61,6 +64,13 @@ struct BatchAdjointArgs {
 bool adjoint_supported(int rhs_id);
 int adjoint_sub_steps(int64_t checkpoint_every);  // M >= K up to 16, else M * M >= K (K at most 256)
 int64_t adjoint_partial_rows(int num_sms);
+// The packed Lorenz RK4 sweeps write one row of kTaskRow doubles per warp task (32 particle
+// pairs), so that a task's sum does not depend on which warp took it: doubles for `capacity`
+// particles (0 for the sweeps whose rows belong to blocks).
+constexpr int kTaskRow = 4;
+inline size_t adjoint_task_doubles(int rhs_id, int method, int64_t capacity) {
+    return rhs_id == FF_RHS_LORENZ && method == FF_RK4 ? (size_t)((capacity + 63) / 64) * kTaskRow : 0;
+}
 // Threads of the HH x 3 sweep (standalone or batched): each needs a scratch area of
 // (largest chunk) x adjoint_scratch_floats_per_step floats; 0 for the systems whose
 // sweeps keep their states on chip.

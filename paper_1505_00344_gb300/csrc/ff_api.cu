@@ -128,7 +128,12 @@ ff_status ff_create_system(int rhs_id, int dim, const double* params, int n_para
     const size_t plane_bytes = sizeof(float) * (size_t)s->pitch;
     e = cudaMalloc(&s->d_state, plane_bytes * dim);
     if (e == cudaSuccess && (flags & FF_FLAG_KAHAN)) e = cudaMalloc(&s->d_comp, plane_bytes * dim);
-    if (e == cudaSuccess) e = cudaMalloc(&s->d_counter, sizeof(unsigned long long));
+    const size_t counters = sizeof(unsigned long long) + sizeof(ff::WorkQueue);
+    if (e == cudaSuccess) e = cudaMalloc(&s->d_counter, counters);
+    if (e == cudaSuccess) {
+        s->d_queue = reinterpret_cast<ff::WorkQueue*>(s->d_counter + 1);
+        e = cudaMemsetAsync(s->d_counter, 0, counters, s->stream);
+    }
     if (e == cudaSuccess) e = cudaMemsetAsync(s->d_state, 0, plane_bytes * dim, s->stream);
     if (e == cudaSuccess && s->d_comp) e = cudaMemsetAsync(s->d_comp, 0, plane_bytes * dim, s->stream);
     if (e != cudaSuccess) {
@@ -444,6 +449,7 @@ static ff_status upload_reset_table(ff_system* s) {
 namespace ff {
 void fill_integrate_args(const ff_system* s, double dt, IntegrateArgs* out) {
     IntegrateArgs a{};
+    a.queue = s->d_queue;
     a.x = s->d_state;
     a.comp = s->d_comp;
     a.pparam = s->d_pparam;
@@ -632,7 +638,10 @@ ff_status ff_tape_begin(ff_system* s, int64_t checkpoint_every, int64_t max_step
         s->partial_blocks = ff::adjoint_partial_rows(s->num_sms);
         e = cudaMalloc(&s->d_ckpt, sizeof(float) * (size_t)slots * s->dim * s->pitch);
         if (e == cudaSuccess) e = cudaMalloc(&s->d_chunks, sizeof(ff::AdjChunk) * (size_t)slots);
-        if (e == cudaSuccess) e = cudaMalloc(&s->d_partial, sizeof(double) * (size_t)s->partial_blocks * FF_MAX_PARAMS);
+        size_t partial = (size_t)s->partial_blocks * FF_MAX_PARAMS;
+        const size_t task_rows = ff::adjoint_task_doubles(s->rhs_id, s->method, s->capacity);
+        if (task_rows > partial) partial = task_rows;
+        if (e == cudaSuccess) e = cudaMalloc(&s->d_partial, sizeof(double) * partial);
         if (e == cudaSuccess) e = cudaMalloc(&s->d_dp, sizeof(double) * FF_MAX_PARAMS);
         if (e != cudaSuccess) {
             free_tape(s);
@@ -689,6 +698,7 @@ ff_status ff_backward(ff_system* s, const float* dL_dxT_dev, float* dL_dx0_dev, 
     a.pitch = s->pitch;
     a.n_groups = s->n_groups;
     a.max_chunk = (int)s->tape_every;
+    a.queue = s->d_queue;
     for (int g = 0; g < s->n_groups; ++g) a.gstart[g] = s->groups[g].start;
     // the HH x 3 sweep keeps a chunk of stage points per thread in a scratch area,
     // allocated on first use and kept with the tape

@@ -39,7 +39,33 @@ __device__ __forceinline__ float rcp_ftz(float x) {
     return y;
 }
 
+// Work handed out to warps as they come free.  A persistent grid's scheduler favours its older
+// warps, so equal shares leave some warps done early and the rest alone at the end (11.4 of 16
+// warps of the Lorenz adjoint sweep were active on average).  Each warp takes its own task first
+// and then the next one from the queue; the last warp to find none clears the queue for the
+// next launch, so launches on one stream, also replayed from a graph, share one.
+struct WorkQueue {
+    unsigned next;  // tasks handed out beyond the first of every warp
+    unsigned done;  // warps that found none
+};
+
+// f(task) for the calling warp's tasks of 0 .. n_tasks - 1 (n_tasks < 2^31), all its lanes together.
+template <class F>
+__device__ __forceinline__ void warp_tasks(WorkQueue* queue, int64_t n_tasks, F&& f) {
+    const unsigned warps = gridDim.x * (blockDim.x >> 5), lane = threadIdx.x & 31;
+    // warp-major as warp_major_first: a partial first round spreads over all blocks
+    for (int64_t w = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; w < n_tasks;) {
+        f(w);
+        __syncwarp();
+        unsigned t = 0;
+        if (lane == 0) t = atomicAdd(&queue->next, 1u);
+        w = (int64_t)warps + __shfl_sync(0xffffffffu, t, 0);
+    }
+    if (lane == 0 && atomicInc(&queue->done, warps - 1) == warps - 1) atomicExch(&queue->next, 0u);
+}
+
 struct IntegrateArgs {
+    WorkQueue* queue;      // the system's (kernels that hand out their work)
     float* x;              // state planes
     float* comp;           // Kahan compensation planes (KAHAN only)
     const float* pparam;   // per-particle parameter values (PP only)

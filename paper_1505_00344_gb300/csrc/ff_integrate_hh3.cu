@@ -8,9 +8,11 @@ namespace {
 // Two particles per thread, all three neurons packed across the pair (hh3_rk4_x2_item).
 template <bool PP, bool TAPE>
 __global__ void __launch_bounds__(HH3::MAX_BLOCK / 2, 3) hh3_rk4_x2_kernel(const __grid_constant__ IntegrateArgs a) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t t = warp_major_first(blockIdx.x, gridDim.x); t < a.n_vec; t += stride)
-        hh3_rk4_x2_item<PP, TAPE>(a, t, (int)a.n_steps);
+    // handed out (equal shares: 1,048,576 particles x 200 steps 5,021 us, handed out 4,894 us)
+    warp_tasks(a.queue, (a.n_vec + 31) / 32, [&](int64_t w) {
+        const int64_t t = w * 32 + (threadIdx.x & 31);
+        if (t < a.n_vec) hh3_rk4_x2_item<PP, TAPE>(a, t, (int)a.n_steps);
+    });
 }
 
 // One neuron per lane: lanes 3j, 3j + 1 and 3j + 2 of a warp (j < 10) hold neurons 0, 1 and 2

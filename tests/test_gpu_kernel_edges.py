@@ -310,3 +310,38 @@ def test_batch_tiles_cover_every_particle(counts, tuned):
         y.set_launch(1)
         y.step(4, 0.01)
         np.testing.assert_array_equal(_states(x), _states(y))
+
+
+@pytest.mark.parametrize("n", [25, 130_003])
+def test_handed_out_work_replays_and_is_deterministic(n):
+    """The queue that hands out a launch's tasks is clear for the next one: a captured step
+    replays to the states of the calls, and two sweeps of one tape give the same gradients."""
+    side = torch.cuda.Stream()
+    captured, called = (ff.System("hh3", HH, n, stream=side.cuda_stream) for _ in "ab")
+    for s in (captured, called):
+        s.seed(n, *HH_BOX, +1, 5)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        captured.step(3, 0.01)
+    for _ in range(3):
+        with torch.cuda.stream(side):
+            graph.replay()
+        called.step(3, 0.01)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(_states(captured), _states(called))
+    for rhs, params, box, every in (("lorenz", [10.0, 28.0, 8 / 3], ([-30, -30, 0], [30, 30, 60]), 20),
+                                    ("lorenz", [10.0, 28.0, 8 / 3], ([-30, -30, 0], [30, 30, 60]), 10),
+                                    ("hh3", HH, HH_BOX, 10)):
+        dim = len(box[0])
+        s = ff.System(rhs, params, n, stream=_stream())
+        s.seed(n, *box, +1, 5)
+        s.tape_begin(every, 40)
+        s.step(40, 0.001)
+        lam = torch.randn((dim, n), device="cuda")
+        got = []
+        for _ in range(2):
+            out = torch.empty_like(lam)
+            got.append((s.backward(lam, out, len(params)).copy(), out))
+        np.testing.assert_array_equal(got[0][0], got[1][0])
+        assert torch.equal(got[0][1], got[1][1])
