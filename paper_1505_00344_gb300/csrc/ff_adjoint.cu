@@ -81,7 +81,7 @@ int64_t adjoint_scratch_threads(int rhs_id, int method, bool pp, int num_sms, bo
 cudaError_t launch_adjoint(int rhs_id, int method, bool pp, int m, const AdjointArgs& a0, int num_sms,
                            cudaStream_t s, double* dL_dp_dev, int n_params_kernel) {
     AdjointArgs a = a0;
-    if (adjoint_task_doubles(rhs_id, method, a.n) > 0) a.np_stride = kTaskRow;
+    if (adjoint_task_row(rhs_id, method) > 0) a.np_stride = adjoint_task_row(rhs_id, method);
     const int block = 128;
     int64_t rows = 0;
     cudaError_t e;

@@ -64,12 +64,15 @@ struct BatchAdjointArgs {
 bool adjoint_supported(int rhs_id);
 int adjoint_sub_steps(int64_t checkpoint_every);  // M >= K up to 16, else M * M >= K (K at most 256)
 int64_t adjoint_partial_rows(int num_sms);
-// The packed Lorenz RK4 sweeps write one row of kTaskRow doubles per warp task (32 particle
-// pairs), so that a task's sum does not depend on which warp took it: doubles for `capacity`
-// particles (0 for the sweeps whose rows belong to blocks).
-constexpr int kTaskRow = 4;
+// The sweeps that hand out warp tasks (packed Lorenz RK4: 32 particle pairs; HH x 3: 20 particles)
+// write one row of partial sums per task, so that a sum does not depend on which warp took it.
+// Doubles per row, 0 for the sweeps whose rows belong to blocks; and for `capacity` particles.
+inline int adjoint_task_row(int rhs_id, int method) {
+    return rhs_id == FF_RHS_HH3 ? 16 : (rhs_id == FF_RHS_LORENZ && method == FF_RK4 ? 4 : 0);
+}
 inline size_t adjoint_task_doubles(int rhs_id, int method, int64_t capacity) {
-    return rhs_id == FF_RHS_LORENZ && method == FF_RK4 ? (size_t)((capacity + 63) / 64) * kTaskRow : 0;
+    const int per = rhs_id == FF_RHS_HH3 ? 20 : 64;
+    return (size_t)((capacity + per - 1) / per) * adjoint_task_row(rhs_id, method);
 }
 // Threads of the HH x 3 sweep (standalone or batched): each needs a scratch area of
 // (largest chunk) x adjoint_scratch_floats_per_step floats; 0 for the systems whose

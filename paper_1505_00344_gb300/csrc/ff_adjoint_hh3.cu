@@ -23,7 +23,7 @@
 // The parameter gradient is carried in twelve FP32 sums per neuron and particle
 // over the chunk, from which the sixteen components are formed in FP64 at the
 // chunk's end (each a sum times a parameter constant); the FP64 sums are reduced
-// over particles through per-block partials in a fixed order.
+// over particles through per-task (batched: per-tile) partials in a fixed order.
 #include "ff_adjoint_impl.cuh"
 
 namespace ff {
@@ -478,6 +478,21 @@ __device__ __forceinline__ void gacc_store(SplitShared& sh, double* row) {
     block_sum_to_row<HH3::NP, kSplitBlock / 32>(g, sh.red, row);
 }
 
+// The warp's sums over its lanes' gacc columns to the task's row: lanes q and q + 16 add component
+// q's halves (each starting at its own column, so that the sixteen components' accesses fall in
+// different banks), and the columns are cleared.
+__device__ __forceinline__ void gacc_to_row(SplitShared& sh, double* row) {
+    const int lane = threadIdx.x & 31, q = lane & 15, base = (threadIdx.x & ~31) + (lane & 16);
+    __syncwarp();
+    double v = 0.0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v += sh.gacc[q * kSplitBlock + base + ((i + q) & 15)];
+    v += __shfl_down_sync(0xffffffffu, v, 16);
+    if (lane < 16) row[q] = v;
+    __syncwarp();
+    gacc_clear(sh);
+}
+
 template <int METHOD, bool PP>
 __global__ void __launch_bounds__(kSplitBlock, kSplitMinBlocks) adjoint_hh3_split_kernel(
     const __grid_constant__ AdjointArgs a) {
@@ -487,12 +502,12 @@ __global__ void __launch_bounds__(kSplitBlock, kSplitMinBlocks) adjoint_hh3_spli
     const int64_t T = (int64_t)gridDim.x * blockDim.x;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     unsigned long long* scr = reinterpret_cast<unsigned long long*>(a.scratch) + t;
-    const int64_t n_tasks = (a.n + kWarpParticles - 1) / kWarpParticles;
-    const int64_t warps = (int64_t)gridDim.x * (kSplitBlock / 32);
-    for (int64_t w = (int64_t)blockIdx.x * (kSplitBlock / 32) + (threadIdx.x >> 5); w < n_tasks; w += warps)
+    // 65,537 particles x 60 steps: 511 us in equal shares (two rounds for most warps), 480 handed out
+    warp_tasks(a.queue, (a.n + kWarpParticles - 1) / kWarpParticles, [&](int64_t w) {
         lane_sweep<METHOD, PP>(a, w * kWarpParticles, a.n, scr, T, sh.stage + threadIdx.x, sh.gacc + threadIdx.x,
                                kSplitBlock);
-    gacc_store(sh, a.partial + (int64_t)blockIdx.x * a.np_stride);
+        gacc_to_row(sh, a.partial + w * a.np_stride);
+    });
 }
 
 // Batched form: tiles of up to 80 particles of one member, one tile per block at a time.
@@ -542,12 +557,11 @@ cudaError_t launch_split(const AdjointArgs& a, int num_sms, cudaStream_t s, int6
     int64_t cap = resident / kSplitBlock;
     // room in the scratch: adjoint_scratch_floats_per_step floats per thread and step
     if (cap > a.scratch_threads / kSplitBlock) cap = a.scratch_threads / kSplitBlock;
-    if (cap > 8 * a.max_blocks) cap = 8 * a.max_blocks;  // rows of the partial-sum buffer (one per block)
     const int64_t need = (a.n + kSplitBlockParticles - 1) / kSplitBlockParticles;
     const int grid = (int)(need < cap ? need : cap);
     if (grid < 1 || !a.scratch) return cudaErrorInvalidConfiguration;
     kernel<<<grid, kSplitBlock, sizeof(SplitShared), s>>>(a);
-    *rows = grid;
+    *rows = (a.n + kWarpParticles - 1) / kWarpParticles;  // one per warp task
     return cudaGetLastError();
 }
 
