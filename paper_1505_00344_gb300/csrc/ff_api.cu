@@ -128,7 +128,7 @@ ff_status ff_create_system(int rhs_id, int dim, const double* params, int n_para
     const size_t plane_bytes = sizeof(float) * (size_t)s->pitch;
     e = cudaMalloc(&s->d_state, plane_bytes * dim);
     if (e == cudaSuccess && (flags & FF_FLAG_KAHAN)) e = cudaMalloc(&s->d_comp, plane_bytes * dim);
-    const size_t counters = sizeof(unsigned long long) + sizeof(ff::WorkQueue);
+    const size_t counters = sizeof(unsigned long long) + FF_MAX_GROUPS * sizeof(ff::WorkQueue);
     if (e == cudaSuccess) e = cudaMalloc(&s->d_counter, counters);
     if (e == cudaSuccess) {
         s->d_queue = reinterpret_cast<ff::WorkQueue*>(s->d_counter + 1);

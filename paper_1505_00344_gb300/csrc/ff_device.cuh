@@ -49,12 +49,13 @@ struct WorkQueue {
     unsigned done;  // warps that found none
 };
 
-// f(task) for the calling warp's tasks of 0 .. n_tasks - 1 (n_tasks < 2^31), all its lanes together.
+// f(task) for the calling warp's tasks of 0 .. n_tasks - 1 (n_tasks < 2^31), all its lanes
+// together; the queue serves `blocks` blocks, of which this is number `block`.
 template <class F>
-__device__ __forceinline__ void warp_tasks(WorkQueue* queue, int64_t n_tasks, F&& f) {
-    const unsigned warps = gridDim.x * (blockDim.x >> 5), lane = threadIdx.x & 31;
+__device__ __forceinline__ void warp_tasks(WorkQueue* queue, int64_t n_tasks, unsigned block, unsigned blocks, F&& f) {
+    const unsigned warps = blocks * (blockDim.x >> 5), lane = threadIdx.x & 31;
     // warp-major as warp_major_first: a partial first round spreads over all blocks
-    for (int64_t w = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; w < n_tasks;) {
+    for (int64_t w = (int64_t)(threadIdx.x >> 5) * blocks + block; w < n_tasks;) {
         f(w);
         __syncwarp();
         unsigned t = 0;
@@ -63,9 +64,13 @@ __device__ __forceinline__ void warp_tasks(WorkQueue* queue, int64_t n_tasks, F&
     }
     if (lane == 0 && atomicInc(&queue->done, warps - 1) == warps - 1) atomicExch(&queue->next, 0u);
 }
+template <class F>
+__device__ __forceinline__ void warp_tasks(WorkQueue* queue, int64_t n_tasks, F&& f) {
+    warp_tasks(queue, n_tasks, blockIdx.x, gridDim.x, f);
+}
 
 struct IntegrateArgs {
-    WorkQueue* queue;      // the system's (kernels that hand out their work)
+    WorkQueue* queue;      // the system's, one per group (kernels that hand out their work; ungrouped ones use the first)
     float* x;              // state planes
     float* comp;           // Kahan compensation planes (KAHAN only)
     const float* pparam;   // per-particle parameter values (PP only)

@@ -117,8 +117,7 @@ __global__ void __launch_bounds__(256) reset_pair_kernel(const __grid_constant__
     // draw n of the group's stream is the finaliser of seed + n gamma; particle j's r-th reset
     // takes n = (r count + j) dim + 1, ..., so its next one starts count dim gamma further on
     const uint64_t block_of_draws = (uint64_t)t->count[g] * (uint64_t)D * kSplitMixGamma;
-    const int64_t stride = nb * blockDim.x;
-    for (int64_t it = first + warp_major_first(blockIdx.x - a.gblk[g], nb); it < last; it += stride) {
+    auto item = [&](int64_t it) {
         const int64_t i0 = 2 * it;
         f2 X[D];
 #pragma unroll
@@ -192,6 +191,18 @@ __global__ void __launch_bounds__(256) reset_pair_kernel(const __grid_constant__
         }
         *reinterpret_cast<uint2*>(a.age + i0) = make_uint2(age[0], age[1]);
         *reinterpret_cast<uint2*>(a.resets + i0) = make_uint2(nres[0], nres[1]);
+    };
+    // Wilson-Cowan's items, whose re-draws make them uneven, are handed out (780 -> 760 us); Lorenz's
+    // step constants leave the uniform registers in that loop (330 -> 362 us), so it keeps equal shares
+    const unsigned block = blockIdx.x - a.gblk[g];
+    if constexpr (S::SHIFTED < 0) {
+        warp_tasks(a.queue + g, (last - first + 31) / 32, block, (unsigned)nb, [&](int64_t task) {
+            const int64_t it = first + task * 32 + (threadIdx.x & 31);
+            if (it < last) item(it);
+        });
+    } else {
+        const int64_t stride = nb * blockDim.x;
+        for (int64_t it = first + warp_major_first(block, nb); it < last; it += stride) item(it);
     }
 }
 

@@ -18,7 +18,8 @@ namespace {
 // one-particle stepper's, so ensembles too small to hide it keep that one.  2,097,152
 // particles x 200 steps: 1,267 us one particle per thread, 1,144 us in pairs with two
 // reciprocals a stage, 904 us with one, 860 us with the step loop unrolled twice; four logistics on
-// one reciprocal (920 us) and four particles per thread (925 us) gave nothing.  The exponential
+// one reciprocal (920 us) and four particles per thread (925 us) gave nothing.  With the pairs
+// handed out to warps instead of in equal shares it is 816 us.  The exponential
 // unit is then about three quarters busy, the FP32 pipe 58%.
 struct WCWideConsts {
     f2 aE, bE, cE, aI, bI, cI;      // base-2 exponents of the logistics: aE E + bE I + cE, aI E + bI I + cI
@@ -53,11 +54,11 @@ __global__ void __launch_bounds__(256) wc_rk4_x2u_kernel(const __grid_constant__
         if (q < a.n_groups && (int)blockIdx.x >= a.gblk[q]) g = q;
     const int64_t nb = a.gblk[g + 1] - a.gblk[g];
     const int64_t start = a.gstart[g], end = a.gend[g], pairs = (end - start + 1) / 2;
-    const int64_t stride = nb * blockDim.x, t0 = warp_major_first(blockIdx.x - a.gblk[g], nb);
     WilsonCowanRK4 s;
     s.init(a.gh[g], a.p);
     if (!((wide >> g) & 1u)) {
-        for (int64_t t = t0; t < pairs; t += stride)
+        const int64_t stride = nb * blockDim.x;
+        for (int64_t t = warp_major_first(blockIdx.x - a.gblk[g], nb); t < pairs; t += stride)
             for (int64_t i = start + 2 * t; i < start + 2 * t + 2 && i < end; ++i) {
                 float x[2] = {a.x[i], a.x[a.pitch + i]};
                 run_steps<2, false>(a, (int)a.n_steps, [&]() {
@@ -78,7 +79,9 @@ __global__ void __launch_bounds__(256) wc_rk4_x2u_kernel(const __grid_constant__
     c.h2E = HHPair::k(s.h2 * s.iE); c.h2I = HHPair::k(s.h2 * s.iI);
     c.h6E = HHPair::k(s.h6 * s.iE); c.h6I = HHPair::k(s.h6 * s.iI);
     const f2 two = HHPair::k(2.0f);
-    for (int64_t t = t0; t < pairs; t += stride) {
+    warp_tasks(a.queue + g, (pairs + 31) / 32, blockIdx.x - a.gblk[g], (unsigned)nb, [&](int64_t task) {
+        const int64_t t = task * 32 + (threadIdx.x & 31);
+        if (t >= pairs) return;
         const int64_t i0 = start + 2 * t;
         const bool vec = (start & 1) == 0 && i0 + 1 < end, has1 = i0 + 1 < end;
         float xs[2], ys[2];
@@ -118,7 +121,7 @@ __global__ void __launch_bounds__(256) wc_rk4_x2u_kernel(const __grid_constant__
                 a.x[a.pitch + i0 + 1] = ys[1];
             }
         }
-    }
+    });
 }
 
 }  // namespace

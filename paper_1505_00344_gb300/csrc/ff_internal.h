@@ -71,7 +71,7 @@ struct ff_system {
     bool stepped = false;
     double t_fwd = 0, t_bwd = 0, c_fwd = 0, c_bwd = 0;  // Kahan-summed simulated time
     unsigned long long* d_counter = nullptr;
-    ff::WorkQueue* d_queue = nullptr;  // beside the counter; clear between launches
+    ff::WorkQueue* d_queue = nullptr;  // one per group, beside the counter; clear between launches
     uint32_t* d_stage = nullptr;  // device copy of a host image
     size_t stage_bytes = 0;
     // tiled sprite rendering: per-tile counts / offsets / cursors and the tile lists
