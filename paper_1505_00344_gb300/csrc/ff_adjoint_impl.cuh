@@ -177,12 +177,15 @@ __device__ __forceinline__ void lorenz_shift_stage(const float (&P)[3], const fl
 // jx = J^T v, jp += F_p^T v at the shifted point P with d = y - x there:
 // J^T v = (-s v0 - zt v1 + y v2, s v0 - v1 + x v2, -x v1 - b v2),
 // F_p^T v = ((y - x) v0, x v1, -z v2).
+// Every product wants -v1, so the sweeps carry the y-component of lambda and of the l negated
+// (lam[1], v[1] and the sum jp[1] are minus theirs; jx[1] is not), which saves an operation a product
+// (with the last step of a sub-segment reversed from registers, below: 2,166 -> 2,122 us for
+// 1,048,576 particles x 400 steps).
 __device__ __forceinline__ void lorenz_shift_vjp(const float (&P)[3], float d, const LorenzShiftC& c,
                                                  const float (&v)[3], float (&jx)[3], float* jp) {
-    const float nv1 = __fsub_rn(0.0f, v[1]);
-    jx[0] = fmaf(c.ns, v[0], fmaf(P[2], nv1, __fmul_rn(P[1], v[2])));
-    jx[1] = fmaf(c.s, v[0], fmaf(P[0], v[2], nv1));
-    jx[2] = fmaf(P[0], nv1, __fmul_rn(c.nb, v[2]));
+    jx[0] = fmaf(c.ns, v[0], fmaf(P[2], v[1], __fmul_rn(P[1], v[2])));
+    jx[1] = fmaf(c.s, v[0], fmaf(P[0], v[2], v[1]));
+    jx[2] = fmaf(P[0], v[1], __fmul_rn(c.nb, v[2]));
     jp[0] = fmaf(d, v[0], jp[0]);
     jp[1] = fmaf(P[0], v[1], jp[1]);
     jp[2] = fmaf(__fsub_rn(c.nr, P[2]), v[2], jp[2]);
@@ -202,16 +205,19 @@ __device__ __forceinline__ void lorenz_shift_adj(const float (&x)[3], float (&la
     for (int i = 0; i < 3; ++i) { u[i] = __fmul_rn(c.h6, lam[i]); u2[i] = __fadd_rn(u[i], u[i]); }
     lorenz_shift_vjp(x4, d4, c, u, m, jp);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) { sum[i] = m[i]; l[i] = fmaf(c.h1, m[i], u2[i]); }
+    for (int i = 0; i < 3; ++i) { sum[i] = m[i]; l[i] = fmaf(i == 1 ? c.nh1 : c.h1, m[i], u2[i]); }
     lorenz_shift_vjp(x3, d3, c, l, m, jp);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) { sum[i] = __fadd_rn(sum[i], m[i]); l[i] = fmaf(c.h2, m[i], u2[i]); }
+    for (int i = 0; i < 3; ++i) { sum[i] = __fadd_rn(sum[i], m[i]); l[i] = fmaf(i == 1 ? c.nh2 : c.h2, m[i], u2[i]); }
     lorenz_shift_vjp(x2, d2, c, l, m, jp);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) { sum[i] = __fadd_rn(sum[i], m[i]); l[i] = fmaf(c.h2, m[i], u[i]); }
+    for (int i = 0; i < 3; ++i) { sum[i] = __fadd_rn(sum[i], m[i]); l[i] = fmaf(i == 1 ? c.nh2 : c.h2, m[i], u[i]); }
     lorenz_shift_vjp(x, d1, c, l, m, jp);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) lam[i] = __fadd_rn(lam[i], __fadd_rn(sum[i], m[i]));
+    for (int i = 0; i < 3; ++i) {
+        const float g = __fadd_rn(sum[i], m[i]);
+        lam[i] = i == 1 ? __fsub_rn(lam[i], g) : __fadd_rn(lam[i], g);
+    }
 }
 
 template <class R, int METHOD>
@@ -410,6 +416,8 @@ __device__ __forceinline__ void adjoint_particle(const AdjointArgs& a, int64_t i
     float lam[D];
 #pragma unroll
     for (int k = 0; k < D; ++k) lam[k] = (k < a.dim) ? a.lam_in[k * a.n + i] : 0.0f;
+    constexpr bool kNegY = IsLorenz<R>::value && METHOD == FF_RK4;  // lorenz_shift_vjp's sign of the y-component
+    if constexpr (kNegY) lam[1] = -lam[1];
     const float pv = PP ? a.pparam[i] : 0.0f;
     for (int c = a.n_chunks - 1; c >= 0; --c) {
         const AdjChunk& ch = a.chunks[c];
@@ -460,8 +468,9 @@ __device__ __forceinline__ void adjoint_particle(const AdjointArgs& a, int64_t i
             }
         }
 #pragma unroll
-        for (int q = 0; q < NP; ++q) gacc[q] += (double)jp[q];
+        for (int q = 0; q < NP; ++q) gacc[q] += (double)(kNegY && q == 1 ? -jp[q] : jp[q]);
     }
+    if constexpr (kNegY) lam[1] = -lam[1];
 #pragma unroll
     for (int k = 0; k < D; ++k)
         if (k < a.dim) a.lam_out[k * a.n + i] = lam[k];
@@ -526,6 +535,12 @@ __device__ __forceinline__ f2 mul2a(f2 a, f2 b) {
     return r;
 }
 
+__device__ __forceinline__ f2 neg2(f2 v) {
+    float a, b;
+    unpack2(v, a, b);
+    return pack2(-a, -b);
+}
+
 // LorenzShiftC per lane (lane 0 and lane 1 may differ in r, with a per-particle
 // parameter, and in h, across a group boundary).
 struct LorenzPairS {
@@ -588,13 +603,12 @@ __device__ __forceinline__ void lorenz_stage2(const f2 (&P)[3], const f2 (&x)[3]
     out[2] = fma2(ch, kz, x[2]);
 }
 
-// lorenz_shift_vjp lane by lane (0 - v1 is the scalar's negation, also for a zero)
+// lorenz_shift_vjp lane by lane
 __device__ __forceinline__ void lorenz_vjp2(const f2 (&P)[3], f2 d, const LorenzPairS& c, const f2 (&v)[3],
                                             f2 (&jx)[3], f2 (&jp)[3]) {
-    const f2 nv1 = sub2(pack2(0.0f, 0.0f), v[1]);
-    jx[0] = fma2(c.ns, v[0], fma2(P[2], nv1, mul2a(P[1], v[2])));
-    jx[1] = fma2(c.s, v[0], fma2(P[0], v[2], nv1));
-    jx[2] = fma2(P[0], nv1, mul2a(c.nb, v[2]));
+    jx[0] = fma2(c.ns, v[0], fma2(P[2], v[1], mul2a(P[1], v[2])));
+    jx[1] = fma2(c.s, v[0], fma2(P[0], v[2], v[1]));
+    jx[2] = fma2(P[0], v[1], mul2a(c.nb, v[2]));
     jp[0] = fma2(d, v[0], jp[0]);
     jp[1] = fma2(P[0], v[1], jp[1]);
     jp[2] = fma2(sub2(c.nr, P[2]), v[2], jp[2]);
@@ -612,16 +626,19 @@ __device__ __forceinline__ void lorenz_adj2(const f2 (&x)[3], f2 (&lam)[3], cons
     for (int i = 0; i < 3; ++i) { u[i] = mul2a(c.h6, lam[i]); u2[i] = add2(u[i], u[i]); }
     lorenz_vjp2(x4, d4, c, u, m, jp);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) { sum[i] = m[i]; l[i] = fma2(c.h1, m[i], u2[i]); }
+    for (int i = 0; i < 3; ++i) { sum[i] = m[i]; l[i] = fma2(i == 1 ? c.nh1 : c.h1, m[i], u2[i]); }
     lorenz_vjp2(x3, d3, c, l, m, jp);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) { sum[i] = add2(sum[i], m[i]); l[i] = fma2(c.h2, m[i], u2[i]); }
+    for (int i = 0; i < 3; ++i) { sum[i] = add2(sum[i], m[i]); l[i] = fma2(i == 1 ? c.nh2 : c.h2, m[i], u2[i]); }
     lorenz_vjp2(x2, d2, c, l, m, jp);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) { sum[i] = add2(sum[i], m[i]); l[i] = fma2(c.h2, m[i], u[i]); }
+    for (int i = 0; i < 3; ++i) { sum[i] = add2(sum[i], m[i]); l[i] = fma2(i == 1 ? c.nh2 : c.h2, m[i], u[i]); }
     lorenz_vjp2(x, d1, c, l, m, jp);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) lam[i] = add2(lam[i], add2(sum[i], m[i]));
+    for (int i = 0; i < 3; ++i) {
+        const f2 g = add2(sum[i], m[i]);
+        lam[i] = i == 1 ? sub2(lam[i], g) : add2(lam[i], g);
+    }
 }
 
 // The states of the sub-segment being reversed live in shared memory, one
@@ -663,6 +680,7 @@ __global__ void __launch_bounds__(kLx2Block, 8) adjoint_lorenz_x2_kernel(const _
 #pragma unroll
         for (int k = 0; k < 3; ++k)
             lam[k] = pack2(a.lam_in[k * a.n + i0], has1 ? a.lam_in[k * a.n + i1] : 0.0f);
+        lam[1] = neg2(lam[1]);  // the y-component's sign of lorenz_shift_vjp
         const float pv0 = PP ? a.pparam[i0] : 0.0f, pv1 = (PP && has1) ? a.pparam[i1] : 0.0f;
         for (int c = a.n_chunks - 1; c >= 0; --c) {
             const AdjChunk& ch = a.chunks[c];
@@ -717,14 +735,14 @@ __global__ void __launch_bounds__(kLx2Block, 8) adjoint_lorenz_x2_kernel(const _
             for (int q = 0; q < 3; ++q) {
                 float u, w;
                 unpack2(jp[q], u, w);
-                gacc[q] += (double)u;
-                if (has1) gacc[q] += (double)w;
+                gacc[q] += (double)(q == 1 ? -u : u);
+                if (has1) gacc[q] += (double)(q == 1 ? -w : w);
             }
         }
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             float u, w;
-            unpack2(lam[k], u, w);
+            unpack2(k == 1 ? neg2(lam[k]) : lam[k], u, w);
             a.lam_out[k * a.n + i0] = u;
             if (has1) a.lam_out[k * a.n + i1] = w;
         }
@@ -737,9 +755,8 @@ __global__ void __launch_bounds__(kLx2Block, 8) adjoint_lorenz_x2_kernel(const _
 // Packed-pair sweep for chunks longer than 16 steps: sub-segments of 4 steps
 // whose recomputation also keeps each step's three stage points, so the reverse
 // step applies the four Jacobian products without recomputing them.  Per
-// 64-thread block the 4 steps x (state + 3 stage points) take the 24.6 KB the
-// 16 states of the plain sweep took; the sub-checkpoints (up to 64 per chunk)
-// live in local memory.  The stage points are the ones lorenz_adj2 recomputes,
+// 64-thread block the state and 3 stage points of 3 steps take 18.4 KB (the last step
+// is reversed from registers); the sub-checkpoints (up to 64 per chunk) live in local memory.  The stage points are the ones lorenz_adj2 recomputes,
 // operation for operation, so dL/dx0 is unchanged to the bit.
 // ---------------------------------------------------------------------------
 constexpr int kLx2sSub = 4;      // steps per sub-segment
@@ -786,22 +803,25 @@ __device__ __forceinline__ void lorenz_adj2_given(const f2 (&x)[3], const f2 (&x
     for (int i = 0; i < 3; ++i) { u[i] = mul2a(c.h6, lam[i]); u2[i] = add2(u[i], u[i]); }
     lorenz_vjp2(x4, d4, c, u, m, jp);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) { sum[i] = m[i]; l[i] = fma2(c.h1, m[i], u2[i]); }
+    for (int i = 0; i < 3; ++i) { sum[i] = m[i]; l[i] = fma2(i == 1 ? c.nh1 : c.h1, m[i], u2[i]); }
     lorenz_vjp2(x3, d3, c, l, m, jp);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) { sum[i] = add2(sum[i], m[i]); l[i] = fma2(c.h2, m[i], u2[i]); }
+    for (int i = 0; i < 3; ++i) { sum[i] = add2(sum[i], m[i]); l[i] = fma2(i == 1 ? c.nh2 : c.h2, m[i], u2[i]); }
     lorenz_vjp2(x2, d2, c, l, m, jp);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) { sum[i] = add2(sum[i], m[i]); l[i] = fma2(c.h2, m[i], u[i]); }
+    for (int i = 0; i < 3; ++i) { sum[i] = add2(sum[i], m[i]); l[i] = fma2(i == 1 ? c.nh2 : c.h2, m[i], u[i]); }
     lorenz_vjp2(x, d1, c, l, m, jp);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) lam[i] = add2(lam[i], add2(sum[i], m[i]));
+    for (int i = 0; i < 3; ++i) {
+        const f2 g = add2(sum[i], m[i]);
+        lam[i] = i == 1 ? sub2(lam[i], g) : add2(lam[i], g);
+    }
 }
 
 template <bool PP>
 __global__ void __launch_bounds__(kLx2Block, 8) adjoint_lorenz_x2s_kernel(const __grid_constant__ AdjointArgs a) {
     constexpr int MS = kLx2sSub;
-    __shared__ f2 st[MS][12][kLx2Block];  // per step: the state, then stage points 2, 3, 4
+    __shared__ f2 st[MS - 1][12][kLx2Block];  // per step but the last: the state, then stage points 2, 3, 4
     const int tid = threadIdx.x;
     const int64_t npair = (a.n + 1) / 2;
     // a task is the 32 pairs of a warp (4,194,304 particles x 400 steps: 9,182 us in equal shares,
@@ -822,6 +842,7 @@ __global__ void __launch_bounds__(kLx2Block, 8) adjoint_lorenz_x2s_kernel(const 
 #pragma unroll
         for (int k = 0; k < 3; ++k)
             lam[k] = pack2(a.lam_in[k * a.n + i0], has1 ? a.lam_in[k * a.n + i1] : 0.0f);
+        lam[1] = neg2(lam[1]);  // the y-component's sign of lorenz_shift_vjp
         const float pv0 = PP ? a.pparam[i0] : 0.0f, pv1 = (PP && has1) ? a.pparam[i1] : 0.0f;
         for (int c = a.n_chunks - 1; c >= 0; --c) {
             const AdjChunk& ch = a.chunks[c];
@@ -857,19 +878,26 @@ __global__ void __launch_bounds__(kLx2Block, 8) adjoint_lorenz_x2s_kernel(const 
 #pragma unroll
                 for (int k = 0; k < 3; ++k) x[k] = cpt[sq][k];
 #pragma unroll
-                for (int r = 0; r < MS; ++r) {
-                    if (r < nq) {
+                for (int r = 0; r < MS - 1; ++r) {
+                    if (r + 1 < nq) {
 #pragma unroll
                         for (int k = 0; k < 3; ++k) st[r][k][tid] = x[k];
                         f2 S[9];
-                        lorenz_fwd2_stages(x, cp2, S, r + 1 < nq);
+                        lorenz_fwd2_stages(x, cp2, S, true);
 #pragma unroll
                         for (int k = 0; k < 9; ++k) st[r][3 + k][tid] = S[k];
                     }
                 }
+                // the last step is reversed at once, from registers
+                {
+                    f2 S[9];
+                    lorenz_fwd2_stages(x, cp2, S, false);
+                    const f2 x2[3] = {S[0], S[1], S[2]}, x3[3] = {S[3], S[4], S[5]}, x4[3] = {S[6], S[7], S[8]};
+                    lorenz_adj2_given(x, x2, x3, x4, lam, cp2, jp);
+                }
 #pragma unroll
-                for (int r = MS - 1; r >= 0; --r)
-                    if (r < nq) {
+                for (int r = MS - 2; r >= 0; --r)
+                    if (r + 1 < nq) {
                         f2 xr[3], x2[3], x3[3], x4[3];
 #pragma unroll
                         for (int k = 0; k < 3; ++k) {
@@ -885,14 +913,14 @@ __global__ void __launch_bounds__(kLx2Block, 8) adjoint_lorenz_x2s_kernel(const 
             for (int q = 0; q < 3; ++q) {
                 float u, w;
                 unpack2(jp[q], u, w);
-                gacc[q] += (double)u;
-                if (has1) gacc[q] += (double)w;
+                gacc[q] += (double)(q == 1 ? -u : u);
+                if (has1) gacc[q] += (double)(q == 1 ? -w : w);
             }
         }
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             float u, w;
-            unpack2(lam[k], u, w);
+            unpack2(k == 1 ? neg2(lam[k]) : lam[k], u, w);
             a.lam_out[k * a.n + i0] = u;
             if (has1) a.lam_out[k * a.n + i1] = w;
         }
