@@ -392,8 +392,8 @@ ff_status ff_backward(ff_system* sys, const float* dL_dxT_dev, float* dL_dx0_dev
 /* Batched stepping (not part of the paper): several systems -- each with its
  * own right-hand side, method, parameters, groups and particle count -- advance
  * together.  Members of one family (same right-hand side, method and presence
- * of a per-particle parameter) run in one persistent launch over a table of work tiles, each block taking tiles
- * round-robin; the families are parallel branches of one CUDA graph, captured
+ * of a per-particle parameter) run in one persistent launch whose warps take
+ * 32 work items of one member at a time; the families are parallel branches of one CUDA graph, captured
  * once per step count and replayed by every ff_batch_step with that count.
  * The systems keep owning their state; the batch borrows them until
  * ff_batch_destroy, and they must not be destroyed, re-seeded, taped (other

@@ -1,5 +1,5 @@
 // ff_batch.cu -- many systems stepped together (not part of the paper): one
-// persistent launch per right-hand-side family over a table of work tiles, the
+// persistent launch per right-hand-side family over its members' work items, the
 // families as parallel branches of one CUDA graph, and an autotuner for the
 // launch shape of each family.
 #include <cstdarg>
@@ -18,65 +18,66 @@
 
 namespace ff {
 
-// Work items [first, first + count) of member system `sys` of a family.
-struct BatchTile {
-    int sys;
-    int pad_;
-    int64_t first;
-    int64_t count;
-};
-
 struct BatchArgs {
     const IntegrateArgs* sys;  // per member: the argument block its own ff_step would use
-    const BatchTile* tiles;
-    int n_tiles;
+    const int* task0;          // per member: its first warp task (32 work items); n_members + 1 entries
+    WorkQueue* queue;          // hands out the tasks
+    int n_members;
+    int n_tasks;
     int n_steps;
     float* const* ckpt;  // taped runs: per member, where to store the state before the steps (or NULL)
 };
 
-// Each block takes tiles round-robin; a tile's system (and so its parameters,
-// groups and step sizes) is the same for the whole block.  A family's members
-// either all have a per-particle parameter (PP) or none has.
-template <class R, int METHOD, bool PP, int PPT>
-__global__ void __launch_bounds__(R::MAX_BLOCK, MinBlocks<R>::value) batch_kernel(const __grid_constant__ BatchArgs b) {
-    for (int tile = blockIdx.x; tile < b.n_tiles; tile += gridDim.x) {
-        const BatchTile T = b.tiles[tile];
-        const IntegrateArgs& a = b.sys[T.sys];
-        float* ck = b.ckpt ? b.ckpt[T.sys] : nullptr;
-        for (int64_t t = T.first + threadIdx.x; t < T.first + T.count; t += blockDim.x) {
-            if (ck) {  // checkpoint of a taped chunk: the state this launch starts from
-                const int64_t i0 = t * PPT;
-                for (int k = 0; k < a.dim; ++k) {
-                    float v[PPT];
-                    Vec<PPT>::load(a.x + k * a.pitch + i0, v);
-                    Vec<PPT>::store(ck + k * a.pitch + i0, v);
-                }
-            }
-            integrate_item<R, METHOD, false, PP, PPT, false, false>(a, t, b.n_steps);  // checkpoint written above
+// f(member, item) for the calling warp's work items, 32 consecutive ones of one member at a time
+// as the queue hands them out: members of any size share the launch evenly.  (Against tiles of
+// whole blocks in equal shares: 64 HH3 systems of 16,384 particles 4.12e10 -> 4.24e10
+// particle-steps/s, the 256-system mix 1.03e11 -> 1.06e11.)
+template <class F>
+__device__ __forceinline__ void batch_items(const BatchArgs& b, F&& f) {
+    warp_tasks(b.queue, b.n_tasks, [&](int64_t w) {
+        int lo = 0, hi = b.n_members - 1;  // the last member whose first task is not beyond w
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (b.task0[mid] <= w) lo = mid;
+            else hi = mid - 1;
         }
+        const int64_t t = (w - b.task0[lo]) * 32 + (threadIdx.x & 31);
+        if (t < b.sys[lo].n_vec) f(lo, t);
+    });
+}
+
+// Checkpoint of a taped chunk: the state of PPT particles this launch starts from.
+template <int PPT>
+__device__ __forceinline__ void batch_checkpoint(const IntegrateArgs& a, float* ck, int64_t t) {
+    const int64_t i0 = t * PPT;
+    for (int k = 0; k < a.dim; ++k) {
+        float v[PPT];
+        Vec<PPT>::load(a.x + k * a.pitch + i0, v);
+        Vec<PPT>::store(ck + k * a.pitch + i0, v);
     }
+}
+
+// A family's members either all have a per-particle parameter (PP) or none has.  HH3 at one particle
+// per thread is the shape of batches too small for pairs, where latency counts and not the
+// standalone kernel's occupancy: two blocks' registers instead of three's, which spilled.
+template <class R, int METHOD, bool PP, int PPT>
+__global__ void __launch_bounds__(R::MAX_BLOCK, MinBlocks<R>::value > 1 ? 2 : 1) batch_kernel(const __grid_constant__ BatchArgs b) {
+    batch_items(b, [&](int member, int64_t t) {
+        const IntegrateArgs& a = b.sys[member];
+        if (float* ck = b.ckpt ? b.ckpt[member] : nullptr) batch_checkpoint<PPT>(a, ck, t);
+        integrate_item<R, METHOD, false, PP, PPT, false, false>(a, t, b.n_steps);  // checkpoint written above
+    });
 }
 
 // HH3 RK4 at two particles per thread: all three neurons of a particle pair packed
 // (hh3_rk4_x2_item, bit-identical to one particle per thread), under its own register bound.
 template <bool PP>
 __global__ void __launch_bounds__(HH3::MAX_BLOCK / 2, 3) batch_hh3_x2_kernel(const __grid_constant__ BatchArgs b) {
-    for (int tile = blockIdx.x; tile < b.n_tiles; tile += gridDim.x) {
-        const BatchTile T = b.tiles[tile];
-        const IntegrateArgs& a = b.sys[T.sys];
-        float* ck = b.ckpt ? b.ckpt[T.sys] : nullptr;
-        for (int64_t t = T.first + threadIdx.x; t < T.first + T.count; t += blockDim.x) {
-            if (ck) {  // checkpoint of a taped chunk: the state this launch starts from
-                const int64_t i0 = t * 2;
-                for (int k = 0; k < a.dim; ++k) {
-                    float v[2];
-                    Vec<2>::load(a.x + k * a.pitch + i0, v);
-                    Vec<2>::store(ck + k * a.pitch + i0, v);
-                }
-            }
-            hh3_rk4_x2_item<PP, false>(a, t, b.n_steps);  // checkpoint written above
-        }
-    }
+    batch_items(b, [&](int member, int64_t t) {
+        const IntegrateArgs& a = b.sys[member];
+        if (float* ck = b.ckpt ? b.ckpt[member] : nullptr) batch_checkpoint<2>(a, ck, t);
+        hh3_rk4_x2_item<PP, false>(a, t, b.n_steps);  // checkpoint written above
+    });
 }
 
 template <class R, int METHOD, bool PP>
@@ -125,11 +126,11 @@ struct ff_batch {
         std::vector<int> members;  // indices into systems
         int ppt = 1, block = 256, grid = 1;
         int steps_per_launch = 0;  // 0: one launch per call; else launches of at most this many steps
-        std::vector<ff::BatchTile> tiles;
+        std::vector<int> task0;  // first warp task of each member, and their number
         std::vector<ff::IntegrateArgs> h_sys;
         ff::IntegrateArgs* d_sys = nullptr;
-        ff::BatchTile* d_tiles = nullptr;
-        size_t tiles_cap = 0;
+        int* d_task0 = nullptr;           // device copy, followed by the family's work queue
+        ff::WorkQueue* d_queue = nullptr;
         cudaStream_t side = nullptr;
         cudaEvent_t done = nullptr;
         double tuned_rate = 0.0;  // particle-steps/s of the chosen shape, if tuned
@@ -166,8 +167,8 @@ struct ff_batch {
 
 namespace {
 
-ff_status build_tiles(ff_batch* b, ff_batch::Family& f) {
-    f.tiles.clear();
+// The members' warp tasks and the grid for the family's launch shape.
+ff_status build_tasks(ff_batch* b, ff_batch::Family& f) {
     const void* k = ff::family_kernel(f.rhs_id, f.method, f.ppt, f.pp);
     if (!k) return fail(FF_ERR_INVALID_ARG, "ff_batch: %d particles per thread not available for this system", f.ppt);
     cudaFuncAttributes attr;
@@ -178,37 +179,18 @@ ff_status build_tiles(ff_batch* b, ff_batch::Family& f) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, f.block, 0);
     if (e != cudaSuccess || occ < 1) return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e,
                                                        "ff_batch: occupancy");
-    const int64_t cap = (int64_t)occ * b->num_sms;
-    // Items per thread of a tile: a tile is the grain the blocks are balanced by, so it shrinks
-    // from four items a thread until every resident block would get eight tiles, or to one item.
-    // 100 steps of 24 mixed systems, 1.6M particles: 1,290 -> 1,204 us tuned; of 6 with 35,000:
-    // 280 -> 89 us (four items a thread left most SMs idle); 64 HH3 systems of 16,384: 5% less.
-    int64_t items = 0;
-    for (int m : f.members) items += ((b->systems[m]->n_particles + 3) / 4 * 4) / f.ppt;
-    int64_t per = items / (cap * f.block * 8);
-    per = per < 1 ? 1 : (per > 4 ? 4 : per);
-    const int64_t tile_items = (int64_t)f.block * per;
-    for (int m = 0; m < (int)f.members.size(); ++m) {
-        const ff_system* s = b->systems[f.members[m]];
-        const int64_t n_vec = ((s->n_particles + 3) / 4 * 4) / f.ppt;
-        for (int64_t first = 0; first < n_vec; first += tile_items) {
-            ff::BatchTile t{};
-            t.sys = m;
-            t.first = first;
-            t.count = (n_vec - first < tile_items) ? n_vec - first : tile_items;
-            f.tiles.push_back(t);
-        }
+    f.task0.assign(1, 0);
+    int64_t tasks = 0;
+    for (int m : f.members) {
+        const int64_t n_vec = ((b->systems[m]->n_particles + 3) / 4 * 4) / f.ppt;
+        tasks += (n_vec + 31) / 32;
+        if (tasks > INT32_MAX) return fail(FF_ERR_UNSUPPORTED, "ff_batch: more than 2^31 warps of work in one family");
+        f.task0.push_back((int)tasks);
     }
-    f.grid = (int)((int64_t)f.tiles.size() < cap ? (int64_t)f.tiles.size() : cap);
-    if (f.tiles.size() > f.tiles_cap) {
-        cudaFree(f.d_tiles);
-        f.d_tiles = nullptr;
-        e = cudaMalloc(&f.d_tiles, sizeof(ff::BatchTile) * f.tiles.size());
-        if (e != cudaSuccess) return cuda_fail(e, "ff_batch: tile table");
-        f.tiles_cap = f.tiles.size();
-    }
-    e = cudaMemcpy(f.d_tiles, f.tiles.data(), sizeof(ff::BatchTile) * f.tiles.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return cuda_fail(e, "ff_batch: tile upload");
+    const int64_t cap = (int64_t)occ * b->num_sms, need = (tasks + f.block / 32 - 1) / (f.block / 32);
+    f.grid = (int)(need < cap ? need : cap);
+    e = cudaMemcpy(f.d_task0, f.task0.data(), sizeof(int) * f.task0.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return cuda_fail(e, "ff_batch: task table upload");
     return FF_OK;
 }
 
@@ -227,7 +209,8 @@ ff_status upload_args(ff_batch* b, ff_batch::Family& f, const double* dts) {
 }
 
 cudaError_t launch_family(const ff_batch::Family& f, int n_steps, cudaStream_t st, bool taped = false) {
-    ff::BatchArgs args{f.d_sys, f.d_tiles, (int)f.tiles.size(), n_steps, taped ? f.d_ckpt : nullptr};
+    ff::BatchArgs args{f.d_sys,          f.d_task0, f.d_queue, (int)f.members.size(), f.task0.back(), n_steps,
+                       taped ? f.d_ckpt : nullptr};
     void* params[] = {&args};
     return cudaLaunchKernel(ff::family_kernel(f.rhs_id, f.method, f.ppt, f.pp), dim3(f.grid), dim3(f.block), params, 0, st);
 }
@@ -302,7 +285,7 @@ void destroy_batch(ff_batch* b) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     for (auto& f : b->fams) {
         cudaFree(f.d_sys);
-        cudaFree(f.d_tiles);
+        cudaFree(f.d_task0);
         cudaFree(f.d_ckpt);
         cudaFree(f.d_adj);
         cudaFree(f.d_adj_tiles);
@@ -382,6 +365,12 @@ ff_status ff_batch_create(ff_system* const* systems, int n_systems, void* cuda_s
         f.h_ckpt.assign(f.members.size(), nullptr);
         if (e == cudaSuccess) e = cudaMalloc(&f.d_sys, sizeof(ff::IntegrateArgs) * f.members.size());
         if (e == cudaSuccess) e = cudaMalloc(&f.d_ckpt, sizeof(float*) * f.members.size());
+        const size_t table = (sizeof(int) * (f.members.size() + 1) + 7) / 8 * 8;
+        if (e == cudaSuccess) e = cudaMalloc(&f.d_task0, table + sizeof(ff::WorkQueue));
+        if (e == cudaSuccess) {
+            f.d_queue = reinterpret_cast<ff::WorkQueue*>(reinterpret_cast<char*>(f.d_task0) + table);
+            e = cudaMemset(f.d_queue, 0, sizeof(ff::WorkQueue));
+        }
     }
     if (e != cudaSuccess) {
         ff_status st = cuda_fail(e, "ff_batch_create: resources");
@@ -389,7 +378,7 @@ ff_status ff_batch_create(ff_system* const* systems, int n_systems, void* cuda_s
         return st;
     }
     for (auto& f : b->fams) {
-        ff_status st = build_tiles(b, f);
+        ff_status st = build_tasks(b, f);
         if (st != FF_OK) {
             destroy_batch(b);
             return st;
@@ -650,7 +639,7 @@ ff_status ff_batch_autotune(ff_batch* b, const double* dt, int64_t trial_steps) 
             for (int bi = 0; bi < 4 && e == cudaSuccess && st == FF_OK; ++bi) {
                 f.ppt = ppts[pi];
                 f.block = blocks[bi];
-                st = build_tiles(b, f);
+                st = build_tasks(b, f);
                 if (st != FF_OK) break;
                 if (f.block != blocks[bi]) continue;  // clamped: the same shape as a smaller block
                 st = upload_args(b, f, dt);
@@ -674,7 +663,7 @@ ff_status ff_batch_autotune(ff_batch* b, const double* dt, int64_t trial_steps) 
         f.ppt = best_ppt;
         f.block = best_block;
         f.steps_per_launch = 0;
-        if (st == FF_OK && e == cudaSuccess) st = build_tiles(b, f);
+        if (st == FF_OK && e == cudaSuccess) st = build_tasks(b, f);
         if (st == FF_OK && e == cudaSuccess) st = upload_args(b, f, dt);
         for (int parts = 2; parts <= 4 && st == FF_OK && e == cudaSuccess && trial_steps >= parts; parts *= 2) {
             const int per = (int)((trial_steps + parts - 1) / parts);
@@ -719,9 +708,9 @@ ff_status ff_batch_describe(ff_batch* b, char* text, int text_len) {
     std::string out;
     for (auto& f : b->fams) {
         char line[256];
-        snprintf(line, sizeof(line), "%s/%s%s: %zu systems, %d particles/thread, block %d, grid %d, %zu tiles%s",
+        snprintf(line, sizeof(line), "%s/%s%s: %zu systems, %d particles/thread, block %d, grid %d, %d warp tasks%s",
                  names[f.rhs_id], f.method == FF_RK4 ? "rk4" : "euler", f.pp ? "/per-particle" : "",
-                 f.members.size(), f.ppt, f.block, f.grid, f.tiles.size(), f.tuned_rate > 0 ? "" : " (untuned)");
+                 f.members.size(), f.ppt, f.block, f.grid, f.task0.back(), f.tuned_rate > 0 ? "" : " (untuned)");
         out += line;
         if (f.steps_per_launch > 0) {
             snprintf(line, sizeof(line), ", at most %d steps per launch", f.steps_per_launch);
