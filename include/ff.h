@@ -340,7 +340,9 @@ ff_status ff_last_launch(ff_system* sys, char* kernel, int kernel_len, int* grid
  * pairs, which round differently within the accuracy of single precision, for particles whose
  * whole group (of which the system may hold a slice) has 650 particles per SM or more, untaped,
  * without reset or per-particle parameter, and one particle per thread otherwise;
- * the default is 4 for RK4 on Lorenz, 2 when compensated,
+ * the default is 4 for RK4 on Lorenz (2 at 16 warps per SM where that measured
+ * ahead: below 200 and from 2,500 to 20,000 particles per SM, to 5,000 with a
+ * per-particle parameter; the same bits), 2 when compensated,
  * 2 for plain RK4 on HH3 and WILSON_COWAN, and 1 otherwise; 0 keeps the current value),
  * threads per block (a multiple of 32 up to 1024, default 512 for RK4 on
  * Lorenz and 256 otherwise, 0 keeps the current value; clamped to the kernel's

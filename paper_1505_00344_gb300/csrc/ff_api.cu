@@ -344,6 +344,7 @@ ff_status ff_set_params(ff_system* s, const double* params, int n_params) {
 
 ff_status ff_set_launch(ff_system* s, int ppt, int block, int blocks_per_sm, int64_t max_steps) {
     if (!s) return fail(FF_ERR_INVALID_ARG, "ff_set_launch: system is NULL");
+    const bool keep_ppt = ppt == 0;
     if (ppt == 0) ppt = s->ppt;
     if (block == 0) block = s->block;
     if (ppt != 1 && ppt != 2 && ppt != 4) return fail(FF_ERR_INVALID_ARG, "ff_set_launch: ppt %d not 1, 2 or 4", ppt);
@@ -354,6 +355,7 @@ ff_status ff_set_launch(ff_system* s, int ppt, int block, int blocks_per_sm, int
     if (blocks_per_sm < 0 || blocks_per_sm > 64) return fail(FF_ERR_INVALID_ARG, "ff_set_launch: blocks_per_sm %d", blocks_per_sm);
     if (max_steps < 0) return fail(FF_ERR_INVALID_ARG, "ff_set_launch: max_steps < 0");
     s->ppt = ppt;
+    if (!keep_ppt) s->ppt_default = false;
     s->block = block;
     s->blocks_per_sm = blocks_per_sm;
     s->max_steps = max_steps;
@@ -489,13 +491,37 @@ struct TapePlan {
     int slot0;
 };
 
+// The launch shape of the next integrator launch.  Unless the caller chose, plain RK4 on Lorenz runs
+// two particles per thread (the same bits as four) at 16 warps per SM where that is ahead: in
+// ensembles too small to give every SM sub-partition a warp of four, whose step takes half the
+// instructions, and in those of a few rounds of a persistent grid, whose last round half the
+// work per item evens out (packed pairs fill the FP32 pipe from 16 warps on).  Frames with
+// image on 152 SMs, four / two particles per thread: 16,384 particles x 400 steps 54 / 38 us,
+// 65,536 to 300,000 level, 466,000 281 / 216, 700,000 410 / 316, 1,048,576 x 381 458 / 442,
+// 2,000,003 x 199 468 / 452, 4,194,304 x 95 460 / 466; with a parameter per particle 466,000
+// 276 / 222, 700,000 343 / 323, 910,000 406 / 422, 2,000,003 445 / 462.
+static ff::LaunchShape launch_shape(const ff_system* s) {
+    ff::LaunchShape shape{s->ppt, s->block, s->blocks_per_sm, s->num_sms, s->tape_on};
+    for (int g = 0; g < s->n_groups; ++g)
+        if (s->groups[g].total >= ff::wide_group(s->num_sms)) shape.wide |= 1u << g;
+    if (s->ppt_default && s->rhs_id == FF_RHS_LORENZ && s->method == FF_RK4 && !(s->flags & FF_FLAG_KAHAN)) {
+        const int64_t per_sm = s->n_particles / s->num_sms;
+        if (per_sm < 200 || (per_sm >= 2500 && per_sm < (s->pparam_index >= 0 ? 5000 : 20000))) {
+            shape.ppt = 2;
+            bool aligned = true;
+            for (int g = 0; g < s->n_groups; ++g) aligned = aligned && s->groups[g].start % 2 == 0;
+            if (aligned && s->blocks_per_sm == 0 && s->block == 512) shape.blocks_per_sm = 1;
+        }
+    }
+    return shape;
+}
+
 static ff_status integrate_steps(ff_system* s, int64_t n_steps, double dt, const ff::ViewArgs* fuse = nullptr,
                                  const TapePlan* tape = nullptr) {
     ff::IntegrateArgs a{};
     ff::fill_integrate_args(s, dt, &a);
-    ff::LaunchShape shape{s->ppt, s->block, s->blocks_per_sm, s->num_sms, s->tape_on};
-    for (int g = 0; g < s->n_groups; ++g)
-        if (s->groups[g].total >= ff::wide_group(s->num_sms)) shape.wide |= 1u << g;
+    const ff::LaunchShape shape = launch_shape(s);
+    a.n_vec = a.n_vec * s->ppt / shape.ppt;
     const bool kahan = (s->flags & FF_FLAG_KAHAN) != 0;
     const bool pp = s->pparam_index >= 0;
     if (s->check_every > 0) {
@@ -971,7 +997,7 @@ ff_status ff_step_splat(ff_system* s, int64_t n_steps, double dt, const ff_view*
     probe.n_groups = s->n_groups;
     for (int g = 0; g < s->n_groups; ++g) probe.gstart[g] = s->groups[g].start;
     probe.pidx = s->pparam_index >= 0 ? kernel_param_index(s, s->pparam_index) : -1;
-    ff::LaunchShape shape{s->ppt, s->block, s->blocks_per_sm, s->num_sms};
+    const ff::LaunchShape shape = launch_shape(s);
     const bool fusable = image_is_device && s->rhs_id == FF_RHS_LORENZ && !s->tape_on && s->check_every == 0 &&
                          n_steps > 0 && s->n_particles > 0 && std::isfinite(dt) &&
                          ff::lorenz_uniform_packed(s->method, (s->flags & FF_FLAG_KAHAN) != 0,

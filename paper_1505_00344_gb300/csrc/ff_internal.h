@@ -84,6 +84,7 @@ struct ff_system {
     bool planes_asked = false;   // a picture has asked for them: the next one allocates them
     // launch shape
     int ppt = 1, block = 256, blocks_per_sm = 0;
+    bool ppt_default = true;  // ppt is the default of ff_create_system, not the caller's
     int64_t max_steps = 0;
     // particle reset
     int64_t steps_total = 0;  // steps since the last ff_reset (global step numbers)

@@ -345,3 +345,27 @@ def test_handed_out_work_replays_and_is_deterministic(n):
             got.append((s.backward(lam, out, len(params)).copy(), out))
         np.testing.assert_array_equal(got[0][0], got[1][0])
         assert torch.equal(got[0][1], got[1][1])
+
+
+# The default Lorenz shape by size: either side of each line, groups that start on even and odd
+# particles, with and without a parameter per particle, against four particles per thread.
+@pytest.mark.parametrize("per_sm,extra", [(200, -1), (200, 0), (2500, -1), (2500, 3), (5000, 1), (20000, 0)])
+@pytest.mark.parametrize("odd,parameter", [(0, False), (1, False), (2, True)])
+def test_default_lorenz_shape_keeps_the_bits(per_sm, extra, odd, parameter):
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    first = n // 2 // 4 * 4 + odd
+    view = dict(ndim_view=2, axes=(0, 2), lo=(-30.0, 0.0), hi=(30.0, 60.0), width=320, height=180)
+    out = []
+    for ppt in (0, 4):
+        s = ff.System("lorenz", [10.0, 28.0, 8 / 3], n, stream=_stream())
+        s.seed(first, [-30, -30, 0], [30, 30, 60], +1, 5)
+        s.seed(n - first, [-30, -30, 0], [30, 30, 60], -1, 6)
+        if parameter:
+            s.set_particle_param(1, 20.0, 40.0)
+        s.set_launch(ppt)
+        img = torch.zeros((180, 320), dtype=torch.int32, device="cuda")
+        s.step_splat(7, 0.001, view, img)
+        s.step(5, 0.001)
+        out.append((_states(s), img.cpu().numpy()))
+    np.testing.assert_array_equal(out[0][0], out[1][0])
+    np.testing.assert_array_equal(out[0][1], out[1][1])
