@@ -818,7 +818,12 @@ __device__ __forceinline__ void lorenz_adj2_given(const f2 (&x)[3], const f2 (&x
     }
 }
 
-template <bool PP>
+//
+// UNI: one group, the same parameters and step in every chunk (a.uniform).  The packed constants,
+// 28 registers otherwise, then come from the argument block and stay in uniform registers,
+// which also spares the register file three operands of most packed operations: the FP32 pipe
+// goes from 70 to 74% busy, 2,120 -> 2,018 us for 1,048,576 particles x 400 steps.
+template <bool PP, bool UNI>
 __global__ void __launch_bounds__(kLx2Block, 8) adjoint_lorenz_x2s_kernel(const __grid_constant__ AdjointArgs a) {
     constexpr int MS = kLx2sSub;
     __shared__ f2 st[MS - 1][12][kLx2Block];  // per step but the last: the state, then stage points 2, 3, 4
@@ -849,12 +854,12 @@ __global__ void __launch_bounds__(kLx2Block, 8) adjoint_lorenz_x2s_kernel(const 
             float pa[3], pb[3];
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-                pa[q] = (PP && q == a.pidx) ? pv0 : ch.p[q];
-                pb[q] = (PP && q == a.pidx) ? pv1 : ch.p[q];
+                pa[q] = UNI ? a.uniform_p[q] : (PP && q == a.pidx) ? pv0 : ch.p[q];
+                pb[q] = UNI ? a.uniform_p[q] : (PP && q == a.pidx) ? pv1 : ch.p[q];
             }
             LorenzShiftC ca, cb;
-            ca.init(ch.gh[g0], pa);
-            cb.init(ch.gh[g1], pb);
+            ca.init(UNI ? a.uniform_h : ch.gh[g0], pa);
+            cb.init(UNI ? a.uniform_h : ch.gh[g1], pb);
             const LorenzPairS cp2 = lorenz_pair(ca, cb);
             const int L = ch.n_steps;
             const float* ck = a.ckpt + (int64_t)ch.ckpt * a.dim * a.pitch;

@@ -13,8 +13,9 @@ static cudaError_t launch_lorenz_x2(bool pp, int m, const AdjointArgs& a, int nu
     // sweep with 4-step sub-segments that keep their stage points
     if (a.max_chunk > 16) {
         if (a.max_chunk > kLx2sSub * kLx2sMaxSub) return cudaErrorInvalidValue;
-        return pp ? launch_lorenz_x2_kernel(adjoint_lorenz_x2s_kernel<true>, a, num_sms, s, rows)
-                  : launch_lorenz_x2_kernel(adjoint_lorenz_x2s_kernel<false>, a, num_sms, s, rows);
+        if (a.uniform) return launch_lorenz_x2_kernel(adjoint_lorenz_x2s_kernel<false, true>, a, num_sms, s, rows);
+        return pp ? launch_lorenz_x2_kernel(adjoint_lorenz_x2s_kernel<true, false>, a, num_sms, s, rows)
+                  : launch_lorenz_x2_kernel(adjoint_lorenz_x2s_kernel<false, false>, a, num_sms, s, rows);
     }
     switch (m) {
     case 4: return pp ? launch_lorenz_x2_one<true, 4>(a, num_sms, s, rows) : launch_lorenz_x2_one<false, 4>(a, num_sms, s, rows);

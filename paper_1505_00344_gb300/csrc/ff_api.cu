@@ -725,6 +725,11 @@ ff_status ff_backward(ff_system* s, const float* dL_dxT_dev, float* dL_dx0_dev, 
     a.n_groups = s->n_groups;
     a.max_chunk = (int)s->tape_every;
     a.queue = s->d_queue;
+    a.uniform = s->n_groups == 1 && s->pparam_index < 0;
+    a.uniform_h = s->chunks[0].gh[0];
+    for (int q = 0; q < 3; ++q) a.uniform_p[q] = s->chunks[0].p[q];
+    for (const ff::AdjChunk& c : s->chunks)
+        if (c.gh[0] != a.uniform_h || memcmp(c.p, s->chunks[0].p, sizeof(c.p)) != 0) a.uniform = 0;
     for (int g = 0; g < s->n_groups; ++g) a.gstart[g] = s->groups[g].start;
     // the HH x 3 sweep keeps a chunk of stage points per thread in a scratch area,
     // allocated on first use and kept with the tape

@@ -369,3 +369,25 @@ def test_default_lorenz_shape_keeps_the_bits(per_sm, extra, odd, parameter):
         out.append((_states(s), img.cpu().numpy()))
     np.testing.assert_array_equal(out[0][0], out[1][0])
     np.testing.assert_array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("n", [1, 63, 130, 20_001])
+def test_lorenz_sweep_uniform_and_general_agree(n):
+    """One group with one set of parameters takes the uniform sweep; the same particles as two
+    groups take the general one: the same operations in the same tasks, so the same bits."""
+    def grads(groups):
+        s = ff.System("lorenz", [10.0, 28.0, 8 / 3], n, stream=_stream())
+        first = 0
+        for c in groups:
+            s.seed_slice(c, first, n, [-30, -30, 0], [30, 30, 60], +1, 5)
+            first += c
+        s.tape_begin(33, 100)
+        s.step(100, 0.001)
+        out = torch.empty_like(lam)
+        return s.backward(lam, out, 3).copy(), out.cpu().numpy()
+
+    lam = torch.randn((3, n), device="cuda", generator=torch.Generator(device="cuda").manual_seed(3))
+    one = grads([n])
+    two = grads([n // 3, n - n // 3] if n > 2 else [n])
+    np.testing.assert_array_equal(one[1], two[1])
+    np.testing.assert_array_equal(one[0], two[0])
