@@ -70,7 +70,6 @@ __device__ __forceinline__ void warp_tasks(WorkQueue* queue, int64_t n_tasks, F&
 }
 
 struct IntegrateArgs {
-    WorkQueue* queue;      // the system's, one per group (kernels that hand out their work; ungrouped ones use the first)
     float* x;              // state planes
     float* comp;           // Kahan compensation planes (KAHAN only)
     const float* pparam;   // per-particle parameter values (PP only)
@@ -101,6 +100,8 @@ struct IntegrateArgs {
     float* ckpt;                     // slot q at ckpt + q * ck_stride (dim planes of pitch floats)
     int64_t ck_stride;
     int ck_first, ck_every, ck_slot0, ck_pad_;
+    // kernels that hand out their work: the system's queues, one per group (ungrouped kernels use the first)
+    WorkQueue* queue;
 };
 
 // Checkpoint slot for the state as the launch loads it (a chunk that starts with
