@@ -1142,9 +1142,9 @@ LaunchRecord& last_launch_record();
 // Grid for a persistent launch: enough blocks to cover the work, at most
 // blocks_per_sm (or the occupancy limit) per SM.  The block size is clamped to
 // the kernel's compiled maximum (its launch bound).
-template <class Kernel>
+template <class Kernel, class... First>
 inline cudaError_t persistent_launch(Kernel kernel, const IntegrateArgs& a, const LaunchShape& s0,
-                                     cudaStream_t stream) {
+                                     cudaStream_t stream, First... first) {
     LaunchShape s = s0;
     cudaFuncAttributes attr;
     cudaError_t e = cudaFuncGetAttributes(&attr, kernel);
@@ -1160,7 +1160,7 @@ inline cudaError_t persistent_launch(Kernel kernel, const IntegrateArgs& a, cons
     const int64_t cap = (int64_t)per_sm * s.num_sms;
     const int grid = (int)(need < cap ? need : cap);
     if (grid < 1) return cudaSuccess;
-    kernel<<<grid, s.block, 0, stream>>>(a);
+    kernel<<<grid, s.block, 0, stream>>>(first..., a);
     last_launch_record() = LaunchRecord{(const void*)kernel, grid, s.block};
     return cudaGetLastError();
 }
