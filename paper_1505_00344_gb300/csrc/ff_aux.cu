@@ -434,7 +434,8 @@ __global__ void __launch_bounds__(kSplatBlock) sprite_combine_kernel(const __gri
             const float4 col = p.colour[g];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                hit[k] = hit[k] || wk[k] > 0.f;
+                if (!(wk[k] > 0.f)) continue;  // also where a colour's product with the gain is infinite
+                hit[k] = true;
                 px[k] = make_float4(fmaf(wk[k], col.x, px[k].x), fmaf(wk[k], col.y, px[k].y),
                                     fmaf(wk[k], col.z, px[k].z), fmaf(wk[k], col.w, px[k].w));
             }
