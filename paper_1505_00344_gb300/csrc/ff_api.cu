@@ -760,6 +760,13 @@ ff_status ff_backward(ff_system* s, const float* dL_dxT_dev, float* dL_dx0_dev, 
     return FF_OK;
 }
 
+// While alive, other streams' captures don't restrict this thread's calls (nor do the calls touch them).
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // The device image a render call draws into: the caller's device image, or the
 // system's staging buffer holding (when accumulating) a copy of the caller's host
 // image; cleared first unless accumulating or (clear false) written whole by the caller.
@@ -944,17 +951,22 @@ ff_status ff_project_sprites(ff_system* s, const ff_view* v, const ff_sprite* sp
         pl.stride = (int64_t)pl.wb * pl.hb;
         const size_t need = (size_t)pl.stride * pl.n;
         if (s->planes_cap < need) {
-            cudaFree(s->d_planes);
+            // any other stream that captures in global mode forbids this thread to allocate and loses
+            // its capture by the attempt: stream-ordered calls, which synchronise nothing, outside that rule
+            RelaxedCapture relaxed;
+            if (s->d_planes) e = cudaFreeAsync(s->d_planes, s->stream);
             s->d_planes = nullptr;
             s->planes_cap = 0;
-            if (cudaMalloc(&s->d_planes, sizeof(float4) * need) == cudaSuccess) {
+            if (e == cudaSuccess) e = cudaMallocAsync((void**)&s->d_planes, sizeof(float4) * need, s->stream);
+            if (e == cudaSuccess) {
                 s->planes_cap = need;
                 e = cudaMemsetAsync(s->d_planes, 0, sizeof(float4) * need, s->stream);
-                if (e != cudaSuccess) return cuda_fail(e, "ff_project_sprites: weight planes");
-            } else {
+            } else if (e == cudaErrorMemoryAllocation) {
                 cudaGetLastError();  // no room: the direct technique needs none
+                e = cudaSuccess;
                 planes = false;
             }
+            if (e != cudaSuccess) return cuda_fail(e, "ff_project_sprites: weight planes");
         }
         pl.w = s->d_planes;
     }

@@ -62,3 +62,35 @@ def test_a_colour_that_overflows_stays_on_the_pixels_its_sprites_cover(accumulat
     m = np.isfinite(want)
     # at most 6,040 fragments a pixel: the two orders of FP32 additions differ by less than 2 (f + 8) 2^-24
     np.testing.assert_allclose(got[m], want[m], rtol=2 * 6048 * 2.0 ** -24, atol=0)
+
+
+def test_pictures_leave_another_streams_capture_alone():
+    """A picture that allocates or grows the workspace, drawn while another stream captures in the
+    strictest mode (which refuses calls that may synchronise, and is lost by one): the picture is the direct
+    technique's and the captured graph replays to the steps' states."""
+    mine, other = torch.cuda.Stream(), torch.cuda.Stream()
+    a, b, called = lorenz([3000, 3000], mine.cuda_stream), lorenz([3000], other.cuda_stream), lorenz([3000])
+    ready(a)
+    sprite = dict(radius=12.0, gain=0.5, colours=[[1.0, 0.5, 0.25, 1.0]] * 8)
+    sizes = [(160, 96), (320, 180)]
+    images = [torch.zeros((h, w, 4), device="cuda") for w, h in sizes]
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(other):
+        graph.capture_begin(capture_error_mode="global")
+        try:
+            b.step(3, 0.001)
+            for (w, h), img in zip(sizes, images):
+                a.project_sprites(view(w, h), sprite, img)
+        finally:
+            graph.capture_end()
+        graph.replay()
+    called.step(3, 0.001)
+    torch.cuda.synchronize()
+    x, y = np.empty((3, 3000), np.float32), np.empty((3, 3000), np.float32)
+    b.get_state(x)
+    called.get_state(y)
+    np.testing.assert_array_equal(x, y)
+    for (w, h), img in zip(sizes, images):
+        want = draw(a, view(w, h), dict(sprite, technique=ff.FF_SPRITE_DIRECT), torch.zeros_like(img))
+        np.testing.assert_allclose(img.cpu().numpy(), want, rtol=2 * 6008 * 2.0 ** -24, atol=0)
