@@ -268,11 +268,11 @@ ff_status ff_step_splat(ff_system* sys, int64_t n_steps, double dt, const ff_vie
  *   FF_SPRITE_AUTO    weights summed in one float plane per drawn group, 2 x 2
  *                     pixels to a reduction, and the colours applied once per
  *                     pixel, where that saves enough reductions (many particles
- *                     for the image's size) and from the system's second such
- *                     picture on, which allocates a workspace of 4 bytes per pixel
- *                     and drawn group, kept until the system is destroyed; the
- *                     direct technique elsewhere, under stream capture and where
- *                     the workspace does not fit. */
+ *                     for the image's size) and once the system's pictures could
+ *                     have saved what allocating the workspace costs (its first one,
+ *                     if large): 4 bytes per pixel and drawn group, kept until the
+ *                     system is destroyed; the direct technique elsewhere, under
+ *                     stream capture and where the workspace does not fit. */
 enum { FF_SPRITE_AUTO = 0, FF_SPRITE_DIRECT = 1, FF_SPRITE_TILED = 2 };
 typedef struct ff_sprite {
     float radius;                    /* half-side of the square, pixels: 0 < radius <= 32 */

@@ -926,8 +926,8 @@ ff_status ff_project_sprites(ff_system* s, const ff_view* v, const ff_sprite* sp
             pl.slot[g] = pl.n++;
         }
     }
-    bool planes = sp->technique == FF_SPRITE_AUTO && s->n_particles > 0 &&
-                  ff::sprite_planes_pay(s->n_particles, pl.n, v->width, v->height, sp->radius);
+    const double saving = ff::sprite_planes_saving(s->n_particles, pl.n, v->width, v->height, sp->radius);
+    bool planes = sp->technique == FF_SPRITE_AUTO && s->n_particles > 0 && saving > 0.0;
 
     DeviceScope dev(s->device);
     if (dev.err != cudaSuccess) return cuda_fail(dev.err, "ff_project_sprites: set device");
@@ -940,23 +940,21 @@ ff_status ff_project_sprites(ff_system* s, const ff_view* v, const ff_sprite* sp
         if (e != cudaSuccess) return cuda_fail(e, "ff_project_sprites: capture status");
         planes = cap == cudaStreamCaptureStatusNone;
     }
-    if (planes && !s->planes_asked) {
-        // a system's first picture does not pay for the workspace (about 20 us to allocate and clear)
-        s->planes_asked = true;
-        planes = false;
-    }
     if (planes) {
         pl.wb = (v->width + 1) / 2;
         pl.hb = (v->height + 1) / 2;
         pl.stride = (int64_t)pl.wb * pl.hb;
         const size_t need = (size_t)pl.stride * pl.n;
-        if (s->planes_cap < need) {
+        if (s->planes_cap < need && (s->planes_saving += saving) < ff::kSpritePlanesCost) {
+            planes = false;
+        } else if (s->planes_cap < need) {
             // any other stream that captures in global mode forbids this thread to allocate and loses
             // its capture by the attempt: stream-ordered calls, which synchronise nothing, outside that rule
             RelaxedCapture relaxed;
             if (s->d_planes) e = cudaFreeAsync(s->d_planes, s->stream);
             s->d_planes = nullptr;
             s->planes_cap = 0;
+            s->planes_saving = 0.0;
             if (e == cudaSuccess) e = cudaMallocAsync((void**)&s->d_planes, sizeof(float4) * need, s->stream);
             if (e == cudaSuccess) {
                 s->planes_cap = need;

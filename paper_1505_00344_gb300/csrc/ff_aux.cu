@@ -454,14 +454,14 @@ __global__ void __launch_bounds__(kSplatBlock) sprite_combine_kernel(const __gri
     }
 }
 
-bool sprite_planes_pay(int64_t n, int drawn_groups, int W, int H, float radius) {
+double sprite_planes_saving(int64_t n, int drawn_groups, int W, int H, float radius) {
     // reductions saved: pi R^2 pixels against about (R + 1/2)^2 blocks a sprite; paid: one
     // pass over the planes (4 bytes per pixel and plane, about 5 TB/s) and a launch, in units
     // of the reductions the L2 takes meanwhile.  On 1920 x 1080 with two groups, planes / direct:
     // 300,000 particles of radius 1.5 33 / 32 us, 1,000,000 44 / 64, of radius 1 36 / 38 (the
     // line lies between those).
     const double saved = (double)n * (3.1416 * radius * radius - (radius + 0.5) * (radius + 0.5));
-    return drawn_groups >= 1 && saved > 0.2 * drawn_groups * (double)W * H + 1.0e6;
+    return drawn_groups >= 1 ? saved - 0.2 * drawn_groups * (double)W * H - 1.0e6 : 0.0;
 }
 
 cudaError_t launch_sprites_planes(const SpriteArgs& a, const SpritePlanes& p, int ndim_view, bool accumulate,

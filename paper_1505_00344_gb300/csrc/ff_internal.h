@@ -81,7 +81,7 @@ struct ff_system {
     size_t entries_cap = 0;
     float4* d_planes = nullptr;  // sprite weight planes, zero between calls
     size_t planes_cap = 0;       // 2 x 2 blocks
-    bool planes_asked = false;   // a picture has asked for them: the next one allocates them
+    double planes_saving = 0.0;  // what they would have saved since they last grew (kSpritePlanesCost)
     // launch shape
     int ppt = 1, block = 256, blocks_per_sm = 0;
     bool ppt_default = true;  // ppt is the default of ff_create_system, not the caller's

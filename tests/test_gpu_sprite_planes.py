@@ -1,5 +1,5 @@
-"""Sprites through weight planes (FF_SPRITE_AUTO with enough particles for the image's size, from
-a system's second such picture on) against the direct technique."""
+"""Sprites through weight planes (FF_SPRITE_AUTO with enough particles for the image's size, once
+the system's pictures could have saved what the workspace costs) against the direct technique."""
 import numpy as np
 import pytest
 
@@ -36,10 +36,12 @@ def draw(s, v, sprite, image):
     return image.cpu().numpy()
 
 
-def ready(s):
-    """The system's first picture that asks for the planes is drawn directly; the next ones use them."""
-    img = torch.zeros((10, 10, 4), device="cuda")
-    s.project_sprites(view(10, 10), dict(radius=12.0, colours=[[1.0] * 4] * 8), img)
+def ready(s, width, height):
+    """Pictures of that size until by the size rule the system holds planes for it and all its groups."""
+    saving = s.info()[0] * (np.pi * 32 * 32 - 32.5 ** 2) - 0.2 * 3 * width * height - 1e6
+    img = torch.zeros((height, width, 4), device="cuda")
+    for _ in range(1 + int(2e7 / saving)):
+        s.project_sprites(view(width, height), dict(radius=32.0, colours=[[1.0] * 4] * 8), img)
 
 
 @pytest.mark.parametrize("accumulate", [0, 1])
@@ -48,7 +50,7 @@ def test_a_colour_that_overflows_stays_on_the_pixels_its_sprites_cover(accumulat
     infinite (weight times infinity), all others keep what the other groups give them, and none is NaN --
     on both techniques, which cover the same pixels."""
     s = lorenz([3000, 40, 3000])
-    ready(s)
+    ready(s, 161, 95)
     colours = [[1.0, 0.0, 0.5, 1.0], [3e38, 0.25, 0.0, 3e38], [0.0, 0.3, 0.9, 0.125]]
     out = []
     for technique in (ff.FF_SPRITE_AUTO, ff.FF_SPRITE_DIRECT):
@@ -69,9 +71,8 @@ def test_pictures_leave_another_streams_capture_alone():
     strictest mode (which refuses calls that may synchronise, and is lost by one): the picture is the direct
     technique's and the captured graph replays to the steps' states."""
     mine, other = torch.cuda.Stream(), torch.cuda.Stream()
-    a, b, called = lorenz([3000, 3000], mine.cuda_stream), lorenz([3000], other.cuda_stream), lorenz([3000])
-    ready(a)
-    sprite = dict(radius=12.0, gain=0.5, colours=[[1.0, 0.5, 0.25, 1.0]] * 8)
+    a, b, called = lorenz([6000, 6000], mine.cuda_stream), lorenz([3000], other.cuda_stream), lorenz([3000])
+    sprite = dict(radius=32.0, gain=0.5, colours=[[1.0, 0.5, 0.25, 1.0]] * 8)
     sizes = [(160, 96), (320, 180)]
     images = [torch.zeros((h, w, 4), device="cuda") for w, h in sizes]
     torch.cuda.synchronize()
@@ -93,4 +94,26 @@ def test_pictures_leave_another_streams_capture_alone():
     np.testing.assert_array_equal(x, y)
     for (w, h), img in zip(sizes, images):
         want = draw(a, view(w, h), dict(sprite, technique=ff.FF_SPRITE_DIRECT), torch.zeros_like(img))
-        np.testing.assert_allclose(img.cpu().numpy(), want, rtol=2 * 6008 * 2.0 ** -24, atol=0)
+        np.testing.assert_allclose(img.cpu().numpy(), want, rtol=2 * 12008 * 2.0 ** -24, atol=0)
+
+
+@pytest.mark.parametrize("n,radius,pictures,allocates", [(400_000, 1.5, 3, False), (400_000, 12.0, 1, True)])
+def test_the_workspace_comes_once_it_would_have_paid(n, radius, pictures, allocates):
+    """A system whose pictures save little draws several of them without the workspace (16 bytes a pixel
+    block of 4096 x 2160, 35 MB); one whose first picture saves more than the allocation costs has it at once."""
+    s = lorenz([n])
+    img = torch.zeros((400, 400, 4), device="cuda")
+    big = torch.zeros((2160, 4096, 4), device="cuda")
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    if not allocates:
+        assert 0 < n * (np.pi * radius ** 2 - (radius + 0.5) ** 2) - 0.2 * 400 * 400 - 1e6 < 2e7 / pictures
+    before = free()
+    for _ in range(pictures):
+        s.project_sprites(view(*((4096, 2160) if allocates else (400, 400))), dict(radius=radius, colours=[[1.0] * 4] * 8),
+                          big if allocates else img)
+    assert (before - free() >= 30 * 2 ** 20) == allocates
+    assert allocates or before == free()
