@@ -1,10 +1,11 @@
 """Sprites through weight planes (FF_SPRITE_AUTO with enough particles for the image's size, once
-the system's pictures could have saved what the workspace costs) against the direct technique."""
+the system's pictures could have saved what the workspace costs) against the oracle and the direct technique."""
 import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
 
+import oracle  # noqa: E402
 import paper_1505_00344_gb300 as ff  # noqa: E402
 
 pytestmark = pytest.mark.gpu
@@ -64,6 +65,54 @@ def test_a_colour_that_overflows_stays_on_the_pixels_its_sprites_cover(accumulat
     m = np.isfinite(want)
     # at most 6,040 fragments a pixel: the two orders of FP32 additions differ by less than 2 (f + 8) 2^-24
     np.testing.assert_allclose(got[m], want[m], rtol=2 * 6048 * 2.0 ** -24, atol=0)
+
+
+PICTURES = [(160, 96, 12.0, 0b111, 0), (37, 25, 12.0, 0b111, 0), (161, 95, 20.0, 0b101, 0), (160, 96, 16.0, 0b010, 1),
+            (64, 201, 32.0, 0b111, 1), (1, 1, 32.0, 0b111, 0), (2, 3, 14.5, 0b110, 1), (640, 361, 32.0, 0b001, 0),
+            (160, 96, 12.0, 0b111, 0)]
+
+
+def test_one_system_draws_pictures_of_many_sizes():
+    """Sizes, radii and group masks change from picture to picture on one system, whose workspace serves
+    them all: every picture is the oracle's of that view alone, each channel within (f + 8) 2^-24 of
+    the sum of its f fragments' magnitudes (f additions and the rounding of each contribution), untouched
+    pixels exactly as they were."""
+    counts = [2300, 1900, 2100]
+    s = lorenz(counts)
+    ready(s, 640, 361)
+    n, group = sum(counts), np.repeat(np.arange(3, dtype=np.int32), counts)
+    x = np.empty((3, n), np.float32)
+    s.get_state(x)
+    colours = [[1.0, 0.25, 0.0, 1.0], [0.0, 0.5, 1.0, -0.75], [0.3, -1.0, 0.6, 2.0]]
+    rng = np.random.default_rng(2)
+    for W, H, R, mask, accumulate in PICTURES:
+        drawn = bin(mask).count("1")
+        assert n * (np.pi * R * R - (R + 0.5) ** 2) > 0.2 * drawn * W * H + 1e6  # the planes' size rule
+        v = view(W, H, group_mask=mask, accumulate=accumulate)
+        base = rng.uniform(-1, 1, (H, W, 4)).astype(np.float32)
+        got = draw(s, v, dict(radius=R, gain=0.8, colours=colours), torch.from_numpy(base).cuda()).astype(np.float64)
+        want, absum, frags = oracle.sprites2d(x[0], x[2], v["lo"], v["hi"], W, H, R, 0.8, colours, group=group,
+                                              include=((mask >> group) & 1).astype(np.uint8))
+        base = base * float(accumulate)
+        assert (np.abs(got - base - want) <= (frags[:, :, None] + 8.0) * 2.0 ** -24 * (absum + np.abs(base))).all()
+        np.testing.assert_array_equal(got[frags == 0], base[frags == 0])
+
+
+@pytest.mark.parametrize("radius", [0.95, 1.5])
+def test_small_sprites_of_many_particles_match_the_oracle(radius):
+    """As above for sprites of one to a few pixels, of which it takes many to pay for the planes."""
+    counts = [1_500_000, 5, 1_500_000]
+    s = lorenz(counts)
+    ready(s, 400, 301)
+    n, group = sum(counts), np.repeat(np.arange(3, dtype=np.int32), counts)
+    assert n * (np.pi * radius ** 2 - (radius + 0.5) ** 2) > 0.2 * 3 * 400 * 301 + 1e6
+    x = np.empty((3, n), np.float32)
+    s.get_state(x)
+    colours, v = [[1.0, 0.25, 0.0, 1.0], [0.0, 0.5, 1.0, -0.75], [0.3, -1.0, 0.6, 2.0]], view(400, 301)
+    got = draw(s, v, dict(radius=radius, gain=0.8, colours=colours), torch.zeros((301, 400, 4), device="cuda"))
+    want, absum, frags = oracle.sprites2d(x[0], x[2], v["lo"], v["hi"], 400, 301, radius, 0.8, colours, group=group)
+    assert (np.abs(got.astype(np.float64) - want) <= (frags[:, :, None] + 8.0) * 2.0 ** -24 * absum).all()
+    np.testing.assert_array_equal(got[frags == 0], 0.0)
 
 
 def test_pictures_leave_another_streams_capture_alone():
