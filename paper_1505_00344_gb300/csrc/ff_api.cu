@@ -45,6 +45,7 @@ ff_status fail(ff_status code, const char* fmt, ...) {
 }
 
 ff_status cuda_fail(cudaError_t e, const char* what) {
+    cudaGetLastError();  // reported here: the next call's launch check must not find it again
     if (e == cudaErrorMemoryAllocation)
         return fail(FF_ERR_OOM, "%s: %s", what, cudaGetErrorString(e));
     return fail(FF_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
