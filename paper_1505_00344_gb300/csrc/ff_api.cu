@@ -10,6 +10,7 @@
 #include <new>
 #include <string>
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "ff.h"
@@ -1041,22 +1042,44 @@ ff_status ff_step_splat(ff_system* s, int64_t n_steps, double dt, const ff_view*
     return FF_OK;
 }
 
-// Whether a caller's buffer is plain memory of the system's device, which a kernel may access
-// (not another device's, a mapped host buffer or an unaligned pointer: those take the copy call).
-static bool device_local(const ff_system* s, const void* p) {
+// Whether [p, p + bytes) lies in the one allocation that p points into, as far as the driver knows it.
+static bool one_allocation(const void* p, size_t bytes) {
+    using Range = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const Range range = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found{};
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<Range>(f);
+    }();
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+    if (!range || range(&base, &size, at) != CUDA_SUCCESS) return false;
+    return at >= base && at - base <= size && bytes <= size - (at - base);
+}
+
+// Whether a caller's buffer is plain memory of the system's device that a kernel may access whole (not
+// another device's, a mapped host buffer, an unaligned pointer or a range beyond its allocation:
+// those take the copy call, which checks what it is given).
+static bool device_local(const ff_system* s, const void* p, size_t bytes) {
     if (reinterpret_cast<uintptr_t>(p) & 3u) return false;
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return at.type == cudaMemoryTypeDevice && at.device == s->device;
+    return at.type == cudaMemoryTypeDevice && at.device == s->device && one_allocation(p, bytes);
 }
 
 // dim planes of P floats between the system's state and a caller's [dim][P].
 static cudaError_t copy_state(ff_system* s, float* dst, int64_t dst_pitch, const float* src, int64_t src_pitch,
                               const void* callers, cudaMemcpyKind kind) {
-    if (kind == cudaMemcpyDeviceToDevice && device_local(s, callers))
+    if (kind == cudaMemcpyDeviceToDevice &&
+        device_local(s, callers, sizeof(float) * (size_t)s->n_particles * s->dim))
         return ff::launch_copy_planes(dst, dst_pitch, src, src_pitch, s->n_particles, s->dim, s->num_sms, s->stream);
     return cudaMemcpy2DAsync(dst, sizeof(float) * dst_pitch, src, sizeof(float) * src_pitch,
                              sizeof(float) * s->n_particles, s->dim, kind, s->stream);
