@@ -337,9 +337,8 @@ ff_status ff_last_launch(ff_system* sys, char* kernel, int kernel_len, int* grid
  * 1 or 2, and plain RK4 at 2 runs all three neurons of two particles packed,
  * bit-identical to 1, from 400 particles per SM on (smaller ensembles run one
  * neuron per thread, with the same bits); plain RK4 on WILSON_COWAN at 2 runs packed
- * pairs, which round differently within the accuracy of single precision, for particles whose
- * whole group (of which the system may hold a slice) has 650 particles per SM or more, untaped,
- * without reset or per-particle parameter, and one particle per thread otherwise;
+ * pairs, bit-identical to 1, where some group has 650 particles per SM or more, without reset,
+ * checkpoints or per-particle parameter, and one particle per thread otherwise;
  * the default is 4 for RK4 on Lorenz (2 at 16 warps per SM where that measured
  * ahead: below 200 and from 2,500 to 20,000 particles per SM, to 5,000 with a
  * per-particle parameter; the same bits), 2 when compensated,

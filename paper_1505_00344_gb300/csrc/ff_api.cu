@@ -503,9 +503,7 @@ struct TapePlan {
 // 2,000,003 x 199 468 / 452, 4,194,304 x 95 460 / 466; with a parameter per particle 466,000
 // 276 / 222, 700,000 343 / 323, 910,000 406 / 422, 2,000,003 445 / 462.
 static ff::LaunchShape launch_shape(const ff_system* s) {
-    ff::LaunchShape shape{s->ppt, s->block, s->blocks_per_sm, s->num_sms, s->tape_on};
-    for (int g = 0; g < s->n_groups; ++g)
-        if (s->groups[g].total >= ff::wide_group(s->num_sms)) shape.wide |= 1u << g;
+    ff::LaunchShape shape{s->ppt, s->block, s->blocks_per_sm, s->num_sms};
     if (s->ppt_default && s->rhs_id == FF_RHS_LORENZ && s->method == FF_RK4 && !(s->flags & FF_FLAG_KAHAN)) {
         const int64_t per_sm = s->n_particles / s->num_sms;
         if (per_sm < 200 || (per_sm >= 2500 && per_sm < (s->pparam_index >= 0 ? 5000 : 20000))) {

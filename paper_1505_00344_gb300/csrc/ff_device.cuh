@@ -1090,12 +1090,16 @@ struct LaunchShape {
     int block;
     int blocks_per_sm;  // 0 = occupancy limit
     int num_sms;
-    bool taped = false;  // the steps are taped (with or without a checkpoint in this launch)
-    uint32_t wide = 0;   // groups whose whole group (a slice's too) has wide_group particles or more
 };
 
-// Size from which a whole group counts as wide (Wilson-Cowan's packed pairs are ahead).
-inline int64_t wide_group(int num_sms) { return 650 * (int64_t)num_sms; }
+// The shape with blocks of at most `most` threads.  A limit of blocks per SM keeps its threads: it counts
+// blocks of the block size it came with, at most the 512 of the one-particle kernels.
+inline LaunchShape with_block_of(LaunchShape s, int most) {
+    if (s.block <= most) return s;
+    if (s.blocks_per_sm > 0) s.blocks_per_sm = s.blocks_per_sm * (s.block < 512 ? s.block : 512) / most;
+    s.block = most;
+    return s;
+}
 
 cudaError_t launch_integrate(int rhs_id, int method, bool kahan, bool pp, const IntegrateArgs& a,
                              const LaunchShape& shape, cudaStream_t stream);
@@ -1207,9 +1211,9 @@ inline cudaError_t launch_reset_variants(int method, bool kahan, bool pp, const 
 
 // Deal the persistent grid's blocks out to the groups in proportion to their
 // sizes (at least one block per group) and launch the group-uniform kernel.
-template <class Kernel, class... More>
+template <class Kernel>
 inline cudaError_t uniform_launch(Kernel kernel, const IntegrateArgs& a0, const LaunchShape& s0,
-                                  cudaStream_t stream, More... more) {
+                                  cudaStream_t stream) {
     LaunchShape s = s0;
     cudaFuncAttributes attr;
     cudaError_t e = cudaFuncGetAttributes(&attr, kernel);
@@ -1237,7 +1241,7 @@ inline cudaError_t uniform_launch(Kernel kernel, const IntegrateArgs& a0, const 
         next += (int)nb;
     }
     a.gblk[a.n_groups] = next;
-    kernel<<<next, s.block, 0, stream>>>(a, more...);
+    kernel<<<next, s.block, 0, stream>>>(a);
     last_launch_record() = LaunchRecord{(const void*)kernel, next, s.block};
     return cudaGetLastError();
 }
