@@ -20,7 +20,7 @@
 // from last to first, each on stage points that cp.async copies brought into the
 // lane's shared-memory column while the step before ran, and apply the four
 // vector-Jacobian products, hand-differentiated from Eq. 6-11.
-// The parameter gradient is carried in twelve FP32 sums per neuron and particle
+// The parameter gradient is carried in thirteen FP32 sums per neuron and particle
 // over the chunk, from which the sixteen components are formed in FP64 at the
 // chunk's end (each a sum times a parameter constant); the FP64 sums are reduced
 // over particles through per-task (batched: per-tile) partials in a fixed order.
@@ -127,9 +127,10 @@ __device__ __forceinline__ void lane_fwd(f2 (&X)[5], const LaneC& L, int src0, u
 
 // FP32 sums over a chunk of one neuron lane's parameter contributions (v_V the
 // adjoint of V, w = v_s (1 - s), act the synaptic sigmoid), each with the factor that
-// makes it a gradient component.  The sum of dV/dt v_V, which 1/C's derivative needs, is
-// the currents' own sums times their conductances, formed at the chunk's end.
-enum { A_U, A_NA, A_NAE, A_K, A_KE, A_L, A_SYN, A_SYNE, A_TR, A_TD, A_SG, A_TH, A_N };
+// makes it a gradient component.  A_CUR sums dV/dt v_V, the net current in which the large ionic
+// currents cancel product by product: formed at the chunk's end from their separate sums, 1/C's
+// derivative had 3 to 9 times the rounding error.
+enum { A_U, A_CUR, A_NA, A_NAE, A_K, A_KE, A_L, A_SYN, A_SYNE, A_TR, A_TD, A_SG, A_TH, A_N };
 struct LaneAcc {
     f2 r[A_N];
     __device__ __forceinline__ f2 get(int i) const { return r[i]; }
@@ -218,7 +219,11 @@ __device__ __forceinline__ void lane_vjp(const f2 (&x)[5], f2 others, const f2 (
     const f2 m2 = mulp(m, m), m3 = mulp(m2, m);
     const f2 n2 = mulp(n, n), n3 = mulp(n2, n), n4 = mulp(n2, n2);
     const f2 dNa = sub2(L.c.ENa, V), dK = sub2(L.c.EK, V), dL = sub2(L.c.EL, V), dS = sub2(L.c.Esyn, V);
-    const f2 tna = mulp(mulp(m3, h), vV), tk = mulp(n4, vV), ts = mulp(others, vV);
+    const f2 m3h = mulp(m3, h), tna = mulp(m3h, vV), tk = mulp(n4, vV), ts = mulp(others, vV);
+    f2 cur = fma2(L.c.gLC, dL, L.driveC);
+    cur = fma2(mulp(L.c.gNaC, m3h), dNa, cur);
+    cur = fma2(mulp(L.c.gKC, n4), dK, cur);
+    cur = fma2(mulp(L.c.gsynC, others), dS, cur);
     jv = O::fms(L.c.gLC, vV, jv);
     jv = O::fms(L.c.gsynC, ts, jv);
     jv = O::fms(L.c.gKC, tk, jv);
@@ -231,6 +236,7 @@ __device__ __forceinline__ void lane_vjp(const f2 (&x)[5], f2 others, const f2 (
     syn = mulp(mulp(L.c.gsynC, dS), vV);
     // parameter sums
     acc.add(A_U, vV);
+    acc.fma(A_CUR, cur, vV);
     acc.add(A_NAE, tna);
     acc.fma(A_NA, tna, dNa);
     acc.add(A_KE, tk);
@@ -322,14 +328,12 @@ __device__ __forceinline__ float group_h(const AdjointArgs& a, const AdjChunk& c
 
 // The sixteen parameter components of one particle's chunk sums (one lane of each
 // register of acc), added to gacc (FP64).
-__device__ __forceinline__ void add_chunk_grads(const float (&p)[HH3::NP], int n, float u, float na, float na_e,
-                                                float k, float k_e, float l, float syn, float syn_e, float tr,
-                                                float td, float sg, float th, double* gacc, int bs) {
+__device__ __forceinline__ void add_chunk_grads(const float (&p)[HH3::NP], int n, float u, float cur, float na,
+                                                float na_e, float k, float k_e, float l, float syn, float syn_e,
+                                                float tr, float td, float sg, float th, double* gacc, int bs) {
     const double invC = 1.0 / (double)p[0], inv_tr = 1.0 / (double)p[12], inv_td = 1.0 / (double)p[13];
     double g[HH3::NP];
-    const double cur = (double)p[9 + n] * u + (double)p[1] * na + (double)p[2] * k + (double)p[3] * l +
-                       (double)p[7] * syn;  // C times the sum of dV/dt v_V
-    g[0] = -cur * invC * invC;
+    g[0] = -(double)cur * invC;
     g[1] = (double)na * invC;
     g[2] = (double)k * invC;
     g[3] = (double)l * invC;
@@ -426,8 +430,9 @@ __device__ __forceinline__ void lane_sweep(const AdjointArgs& a, int64_t first, 
                 lane_adj_rk4(stage + half * kStepPoints * bs, bs, lam, L, acc, src0);
             }
         }
-        float u[2], na[2], na_e[2], kk[2], k_e[2], l[2], syn[2], syn_e[2], tr[2], td[2], sg[2], th[2];
+        float u[2], cur[2], na[2], na_e[2], kk[2], k_e[2], l[2], syn[2], syn_e[2], tr[2], td[2], sg[2], th[2];
         unpack2(acc.get(A_U), u[0], u[1]);
+        unpack2(acc.get(A_CUR), cur[0], cur[1]);
         unpack2(acc.get(A_NA), na[0], na[1]);
         unpack2(acc.get(A_NAE), na_e[0], na_e[1]);
         unpack2(acc.get(A_K), kk[0], kk[1]);
@@ -444,7 +449,7 @@ __device__ __forceinline__ void lane_sweep(const AdjointArgs& a, int64_t first, 
             if (e == 0 ? !v0 : !v1) continue;
             float p[HH3::NP];
             lane_params<PP>(a, ch, e == 0 ? i0 : i1, p);
-            add_chunk_grads(p, n, u[e], na[e], na_e[e], kk[e], k_e[e], l[e], syn[e], syn_e[e], tr[e], td[e],
+            add_chunk_grads(p, n, u[e], cur[e], na[e], na_e[e], kk[e], k_e[e], l[e], syn[e], syn_e[e], tr[e], td[e],
                             sg[e], th[e], gacc, bs);
         }
     }
