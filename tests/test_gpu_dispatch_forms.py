@@ -9,9 +9,8 @@ import paper_1505_00344_gb300 as ff  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 WC = [16.0, 12.0, 15.0, 3.0, 1.25, 0.0, 1.0, 1.0, 1.0, 4.0]
-BOX = {"wilson_cowan": ([0, 0], [1, 1])}
-PARAMS = {"wilson_cowan": WC}
-
+BOX = {"wilson_cowan": ([0, 0], [1, 1]), "lorenz": ([-30, -30, 0], [30, 30, 60])}
+PARAMS = {"wilson_cowan": WC, "lorenz": [10.0, 28.0, 8 / 3]}
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -74,3 +73,47 @@ def test_wilson_cowan_pairs_keep_the_one_particle_bits(small, first):
             out.append(states(s))
         for x in out[1:]:
             np.testing.assert_array_equal(out[0], x)
+
+
+# The launch of the default shape where particles reset, or where sigma or beta is taken per particle,
+# in the range where two particles per thread at 16 warps per SM run otherwise.
+@pytest.mark.parametrize("form", ["reset", "reset, r each", "sigma each", "beta each"])
+def test_default_lorenz_shape_of_other_kernels_fills_the_gpu(form):
+    """The one-block shape belongs to the group-uniform packed kernel: every other launch has the grid and
+    block that a caller gets who asks for four particles per thread, and the same states."""
+    n = 3000 * sms() + 5
+    out = []
+    for ppt in (0, 4):
+        s = system("lorenz", 4 * (n // 8), n - 4 * (n // 8))
+        s.set_launch(ppt)
+        if form != "reset":
+            s.set_particle_param({"reset, r each": 1, "sigma each": 0, "beta each": 2}[form], 2.0, 12.0)
+        if "reset" in form:
+            s.set_reset([-20, -25, 2], [20, 25, 45], 0.02, 1)
+        s.step(9, 0.004)
+        out.append((s.last_launch(), states(s)))
+    np.testing.assert_array_equal(out[0][1], out[1][1])
+    a, b = out[0][0], out[1][0]
+    assert (a["grid"], a["block"]) == (b["grid"], b["block"])
+
+
+# Resetting pairs with several rounds of work per warp, Lorenz at the default shape's ranges.
+@pytest.mark.parametrize("name,per_sm", [("lorenz", 150), ("lorenz", 3000), ("lorenz", 9000), ("wilson_cowan", 6000)])
+def test_large_resetting_ensembles_match_their_parts(name, per_sm):
+    """An ensemble's states, ages and reset counts are those of its slices of up to 1,000 particles per SM
+    run alone, bit for bit."""
+    n, lim = per_sm * sms() + 3, {"lorenz": ([-20, -25, 2], [20, 25, 45]),
+                                  "wilson_cowan": ([0.1, 0.05], [0.9, 0.95])}[name]
+
+    def run(first, count):
+        s = ff.System(name, PARAMS[name], count, stream=torch.cuda.current_stream().cuda_stream)
+        s.seed_slice(count, first, n, *BOX[name], 1, 40)
+        s.set_reset(*lim, 0.05, 2)
+        s.step(21, 0.01)
+        age, res = (np.empty(count, np.uint32) for _ in "ab")
+        s.get_reset_state(age, res)
+        return np.concatenate([states(s).view(np.uint32), age[None], res[None]])
+
+    whole, part = run(0, n), 1000 * sms() + 1
+    for first in range(0, n, part):
+        np.testing.assert_array_equal(run(first, min(part, n - first)), whole[:, first:first + part])
