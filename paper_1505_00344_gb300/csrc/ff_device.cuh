@@ -1093,11 +1093,11 @@ struct LaunchShape {
 };
 
 // The shape with blocks of at most `most` threads.  A limit of blocks per SM keeps its threads: it counts
-// blocks of the block size it came with, at most the 512 of the one-particle kernels.
-inline LaunchShape with_block_of(LaunchShape s, int most) {
-    if (s.block <= most) return s;
-    if (s.blocks_per_sm > 0) s.blocks_per_sm = s.blocks_per_sm * (s.block < 512 ? s.block : 512) / most;
-    s.block = most;
+// blocks of the block size it came with, at most that of the system's one-particle kernel.
+inline LaunchShape with_block_of(LaunchShape s, int most, int one_particle = 512) {
+    const int block = s.block < one_particle ? s.block : one_particle;
+    if (s.blocks_per_sm > 0 && block > most) s.blocks_per_sm = s.blocks_per_sm * block / most;
+    if (s.block > most) s.block = most;
     return s;
 }
 

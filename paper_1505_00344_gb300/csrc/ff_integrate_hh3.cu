@@ -128,7 +128,8 @@ cudaError_t lane_launch_one(const IntegrateArgs& a, const LaunchShape& s, cudaSt
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, 32, 0);
     if (e != cudaSuccess) return e;
     if (occ < 1) return cudaErrorInvalidConfiguration;
-    const int per_sm = (s.blocks_per_sm > 0 && s.blocks_per_sm < occ) ? s.blocks_per_sm : occ;
+    const int limit = with_block_of(s, 32, HH3::MAX_BLOCK).blocks_per_sm;  // the caller's, in warps
+    const int per_sm = (limit > 0 && limit < occ) ? limit : occ;
     const int64_t need = (a.n_vec + 10 * PER - 1) / (10 * PER), cap = (int64_t)per_sm * s.num_sms;
     const int grid = (int)(need < cap ? need : cap);
     if (grid < 1) return cudaSuccess;

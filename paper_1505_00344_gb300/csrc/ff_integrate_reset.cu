@@ -162,7 +162,7 @@ bool reset_pairs(int rhs_id, int method, bool kahan, bool pp, const IntegrateArg
 }
 
 cudaError_t launch_reset_pairs(int rhs_id, const IntegrateArgs& a, const LaunchShape& shape, cudaStream_t stream) {
-    LaunchShape s = shape;
+    LaunchShape s = with_block_of(shape, 256);
     s.ppt = 2;
     if (rhs_id == FF_RHS_WILSON_COWAN) return uniform_launch(reset_pair_kernel<WilsonCowanPair>, a, s, stream);
     return uniform_launch(reset_pair_kernel<LorenzPair>, a, s, stream);

@@ -9,8 +9,10 @@ import paper_1505_00344_gb300 as ff  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 WC = [16.0, 12.0, 15.0, 3.0, 1.25, 0.0, 1.0, 1.0, 1.0, 4.0]
-BOX = {"wilson_cowan": ([0, 0], [1, 1]), "lorenz": ([-30, -30, 0], [30, 30, 60])}
-PARAMS = {"wilson_cowan": WC, "lorenz": [10.0, 28.0, 8 / 3]}
+HH = [1.0, 120.0, 36.0, 0.3, 50.0, -77.0, -54.4, 0.5, -80.0, 8.0, 12.0, 10.0, 0.1, 10.0, 0.5, -20.0]
+BOX = {"wilson_cowan": ([0, 0], [1, 1]), "lorenz": ([-30, -30, 0], [30, 30, 60]),
+       "hh3": ([-80.0, 0, 0, 0, 0] * 3, [40.0, 1, 1, 1, 1] * 3)}
+PARAMS = {"wilson_cowan": WC, "lorenz": [10.0, 28.0, 8 / 3], "hh3": HH}
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -117,3 +119,26 @@ def test_large_resetting_ensembles_match_their_parts(name, per_sm):
     whole, part = run(0, n), 1000 * sms() + 1
     for first in range(0, n, part):
         np.testing.assert_array_equal(run(first, min(part, n - first)), whole[:, first:first + part])
+
+
+# A caller's limit of blocks per SM, which counts blocks of the block size it goes with.
+@pytest.mark.parametrize("name,n,blocks,block,reset", [
+    ("hh3", 12_345, 1, 0, False), ("hh3", 25_001, 2, 96, False), ("hh3", 50_000, 1, 128, False),
+    ("lorenz", 400_001, 1, 0, True), ("wilson_cowan", 400_001, 1, 512, True), ("wilson_cowan", 400_001, 1, 512, False),
+    ("wilson_cowan", 400_001, 3, 0, False), ("wilson_cowan", 400_001, 1, 1024, True)])
+def test_a_limit_of_blocks_per_sm_keeps_its_threads(name, n, blocks, block, reset):
+    """Whatever kernel runs, it has as many threads per SM as the caller's limit gives (blocks times the block
+    size, at most the 512 or 256 of the system's one-particle kernel), if it has the work, and no more."""
+    s = system(name, n)
+    s.set_launch(0, block, blocks)
+    if reset:
+        s.set_reset([v - 1 for v in BOX[name][0]], [v + 1 for v in BOX[name][1]], 0.0, 1)
+    s.step(2, 0.001)
+    launch = s.last_launch()
+    most = 256 if name == "hh3" else 512
+    size = min(block or (512 if name == "lorenz" else 256), most)
+    limit = blocks * size * sms()
+    pairs, lanes = ("x2" in launch["kernel"] or "pair" in launch["kernel"]), "lane_integrate" in launch["kernel"]
+    work = (n + 19) // 20 * 32 if lanes else ((n + 1) // 2 if pairs else n)  # lanes: up to 20 particles a warp
+    threads = launch["grid"] * launch["block"]
+    assert min(limit, work) <= threads <= max(limit, work + launch["block"] - 1), launch
