@@ -20,7 +20,10 @@
  *     are only borrowed for the duration of the call.
  *   - Streams: all device work of a system is enqueued on the CUDA stream
  *     given at creation (NULL = the legacy default stream).  Calls return after
- *     enqueueing unless documented as synchronising.
+ *     enqueueing unless documented as synchronising.  A graph captured from a
+ *     system's calls may be replayed on another stream only in order with the
+ *     system's other work: they share its state and the queues that hand out
+ *     a launch's work, which overlapping launches would leave wrong.
  *   - Device: a system is bound to the device that was current when it was
  *     created; every call makes that device current for its own work and
  *     restores the caller's device before returning.
@@ -238,8 +241,8 @@ ff_status ff_project_splat(ff_system* sys, const ff_view* view, uint32_t* image,
 /* One frame: exactly ff_step(n_steps, dt) followed by
  * ff_project_splat(view, image, image_is_device), with the same results.  When
  * the group-uniform packed Lorenz kernel runs (plain RK4, 2 or 4 particles per
- * thread, 4-aligned groups, per-particle parameter absent or r, no reset, no
- * tape, device image) the projection and splat are fused into the last
+ * thread, groups that start on a multiple of that, per-particle parameter absent
+ * or r, no reset, no tape, device image) the projection and splat are fused into the last
  * integrator launch, which counts each particle from the registers that hold
  * its final state; otherwise the two calls run one after the other.  Errors:
  * those of ff_step and ff_project_splat. */
@@ -348,7 +351,8 @@ ff_status ff_last_launch(ff_system* sys, char* kernel, int kernel_len, int* grid
  * maximum, 512 for the 2- and 3-dimensional systems and 256 for LINEAR and
  * HH3, and narrowed in whole warps when the particles would not give every SM
  * a block, so that a small ensemble spreads over all SMs), resident blocks per
- * SM of the persistent grid (0 = as many as fit), and the most steps per
+ * SM of the persistent grid (0 = as many as fit; kernels with smaller blocks run as
+ * many threads), and the most steps per
  * launch (0 = all steps of an ff_step call in one launch; launches are also
  * split at 2^30 steps).  Errors: FF_ERR_INVALID_ARG for values out of range. */
 ff_status ff_set_launch(ff_system* sys, int particles_per_thread, int block, int blocks_per_sm,
@@ -401,7 +405,8 @@ ff_status ff_backward(ff_system* sys, const float* dL_dxT_dev, float* dL_dx0_dev
  * than by ff_batch_tape_begin) or given a particle reset, and must keep or
  * lack their per-particle parameter meanwhile (ff_batch_step then returns
  * FF_ERR_STATE).
- * Members run the scalar integrator (no packed Lorenz kernel, no fused splat).
+ * Members run the one-particle steppers (HH3 RK4 also in particle pairs; no packed
+ * Lorenz or Wilson-Cowan kernel, no fused splat), with the bits of their own steps.
  *
  * ff_batch_create: systems on one device, each with particles, no Kahan flag,
  *   no reset, no tape; cuda_stream orders the batch's work (NULL = legacy
@@ -416,7 +421,7 @@ ff_status ff_backward(ff_system* sys, const float* dL_dxT_dev, float* dL_dx0_dev
  *   own data for trial_steps steps (twice), keeps the fastest, then times the
  *   same trial split into 2 and 4 launches (steps per launch) and keeps a split
  *   if it is faster; restores the members' states exactly.  Synchronises.
- * ff_batch_describe: one line per family: members, launch shape, tiles, tuned
+ * ff_batch_describe: one line per family: members, launch shape, warp tasks, tuned
  *   rate (NUL-terminated, truncated to text_len).
  *
  * Batched gradients.  ff_batch_tape_begin starts every member's tape

@@ -38,7 +38,7 @@ struct AdjointArgs {
     int64_t gstart[FF_MAX_GROUPS];
     int uniform;              // one group, and every chunk has the parameters and step below
     float uniform_h, uniform_p[3];  // (Lorenz: the first three)
-    WorkQueue* queue;         // packed Lorenz sweeps: hands out their warp tasks
+    WorkQueue* queue;         // Lorenz RK4 and HH x 3 sweeps: hands out their warp tasks
     float* scratch;           // HH x 3 sweep: one chunk of stage points per thread (a neuron of two particles)
     int64_t scratch_threads;  // threads the scratch has room for (see adjoint_scratch_floats_per_step)
 };

@@ -662,8 +662,7 @@ __global__ void __launch_bounds__(kLx2Block, 8) adjoint_lorenz_x2_kernel(const _
     __shared__ f2 st[M][3][kLx2Block];
     const int tid = threadIdx.x;
     const int64_t npair = (a.n + 1) / 2;
-    // a task is the 32 pairs of a warp (4,194,304 particles x 400 steps: 9,182 us in equal shares,
-    // 8,605 us handed out; 262,144: 723 and 633)
+    // a task is the 32 pairs of a warp (adjoint_lorenz_x2s_kernel)
     warp_tasks(a.queue, (npair + 31) / 32, [&](int64_t task) {
         double gacc[3] = {0.0, 0.0, 0.0};
         const int64_t t = task * 32 + (tid & 31);

@@ -86,7 +86,7 @@ __device__ __forceinline__ float draw_value(uint64_t z, const DrawBox& b) {
     const float k = (float)(uint32_t)(z >> 40);  // 24 bits: exact
     const float ph = __fmul_rn(k, b.wh);
     const float pl = fmaf(k, b.wl, fmaf(k, b.wh, -ph));  // k * width / 2^24 = ph + pl
-    const float s = __fadd_rn(b.lh, ph);                 // lh + ph = s + e exactly
+    const float s = __fadd_rn(b.lh, ph);                 // lh + ph = s + e exactly (Knuth's two-sum)
     const float v = __fsub_rn(s, b.lh);
     const float e = __fadd_rn(__fsub_rn(b.lh, __fsub_rn(s, v)), __fsub_rn(ph, v));
     const float t = __fadd_rn(e, __fadd_rn(b.ll, pl));
