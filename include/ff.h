@@ -343,8 +343,8 @@ ff_status ff_last_launch(ff_system* sys, char* kernel, int kernel_len, int* grid
  * pairs, bit-identical to 1, where some group has 650 particles per SM or more, without reset,
  * checkpoints or per-particle parameter, and one particle per thread otherwise;
  * the default is 4 for RK4 on Lorenz (2 at 16 warps per SM where that measured
- * ahead: below 200 and from 2,500 to 20,000 particles per SM, to 5,000 with a
- * per-particle parameter; the same bits), 2 when compensated,
+ * ahead: below 200 particles per SM, and from 2,500 to 20,000 with groups that start on
+ * even particles, to 5,000 with r per particle; not with reset; the same bits), 2 when compensated,
  * 2 for plain RK4 on HH3 and WILSON_COWAN, and 1 otherwise; 0 keeps the current value),
  * threads per block (a multiple of 32 up to 1024, default 512 for RK4 on
  * Lorenz and 256 otherwise, 0 keeps the current value; clamped to the kernel's
