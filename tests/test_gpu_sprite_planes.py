@@ -160,6 +160,8 @@ def test_the_workspace_comes_once_it_would_have_paid(n, radius, pictures, alloca
 
     if not allocates:
         assert 0 < n * (np.pi * radius ** 2 - (radius + 0.5) ** 2) - 0.2 * 400 * 400 - 1e6 < 2e7 / pictures
+    # (the direct kernel's first launch loads its code)
+    s.project_sprites(view(400, 400), dict(radius=1.0, colours=[[1.0] * 4] * 8, technique=ff.FF_SPRITE_DIRECT), img)
     before = free()
     for _ in range(pictures):
         s.project_sprites(view(*((4096, 2160) if allocates else (400, 400))), dict(radius=radius, colours=[[1.0] * 4] * 8),
